@@ -6,6 +6,7 @@
 
 #include <type_traits>
 
+#include "kmc_pair.cuh"
 #include "kmc_stage.cuh"
 #include "kmc_types.h"
 
@@ -91,31 +92,23 @@ struct Prec<double> {
   __device__ static double div(double a, double b) { return a / b; }
   __device__ static double theta(int j) { return g_theta_d[j]; }
   __device__ static double2 sc(int j) { return g_sc_d[j]; }
-  // Taylor series to d^9 / d^10: truncation below 1e-24 for d <= 2 pi / 200
+  // Taylor series to d^7 / d^8: the next terms are below 8.3e-20 and 2.6e-22
+  // for d <= 2 pi / 200, a thousandth of the rounding of the sums
   __device__ static void sincos_small(double d, double &s, double &c) {
     const double d2 = d * d;
-    s = d * fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0),
-                        -1.0 / 6.0),
-                1.0);
-    c = fma(d2,
-            fma(d2, fma(d2, fma(d2, fma(d2, -1.0 / 3628800.0, 1.0 / 40320.0), -1.0 / 720.0),
-                        1.0 / 24.0),
-                -0.5),
-            1.0);
+    s = d * fma(d2, fma(d2, fma(d2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), 1.0);
+    c = fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 40320.0, -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
   }
 };
 
 // Copy of the grid of step iv in shared memory, filled by every block at its
 // start (the pair loop hides the loads); the scan reads one node per warp
 // (a broadcast), Newton one node per thread.
-template <typename R>
-struct ScanPairs {};
-template <>
-struct ScanPairs<float> {
-  float ss[kGridPad], cc[kGridPad];  // g_ss_f, g_cc_f
+struct ScanPairs {
+  float ss[kGridPad], cc[kGridPad];  // g_ss_f, g_cc_f (both precisions scan in FP32)
 };
 template <typename R>
-struct GridTables : ScanPairs<R> {
+struct GridTables : ScanPairs {
   typename std::conditional<std::is_same<R, float>::value, float2, double2>::type sc[kGrid];
   R th[kGrid];
   __device__ void load() {
@@ -123,16 +116,14 @@ struct GridTables : ScanPairs<R> {
       sc[j] = Prec<R>::sc(j);
       th[j] = Prec<R>::theta(j);
     }
-    if constexpr (std::is_same<R, float>::value) {
-      for (int j = threadIdx.x; j < kGridPad; j += blockDim.x) {
-        this->ss[j] = g_ss_f[j];
-        this->cc[j] = g_cc_f[j];
-      }
+    for (int j = threadIdx.x; j < kGridPad; j += blockDim.x) {
+      ss[j] = g_ss_f[j];
+      cc[j] = g_cc_f[j];
     }
   }
 };
 static_assert(sizeof(GridTables<float>::sc) % 16 == 0 && sizeof(GridTables<float>::th) % 16 == 0 &&
-                  sizeof(ScanPairs<float>::ss) % 16 == 0 && sizeof(ScanPairs<float>) % 16 == 0,
+                  sizeof(ScanPairs::ss) % 16 == 0 && sizeof(ScanPairs) % 16 == 0,
               "the FP32 tables are copied in bulk");
 
 // de/dth of Eq. 2 at (sin, cos) = (s, c): s (2k c + b cos phi) - b sin phi c,
@@ -202,6 +193,161 @@ __device__ __forceinline__ R refine_in_cell(const Profile<R> &pf, R S0, R C0, R 
   s_out = fma(S0, cd, C0 * sd);
   c_out = fma(C0, cd, -S0 * sd);
   return x;
+}
+
+// FP64 root of de/dth inside grid cell [theta_j, theta_j + h] (left_neg: de/dth
+// is negative at theta_j), as offset from theta_j; (S0, C0) = sin, cos of
+// theta_j, (S0f, C0f) the same in FP32. FP64 instructions issue at 1/64 of the
+// FP32 rate here, so the search runs in FP32 until its rounding (about 1e-8
+// rad from the cell's middle in three Newton steps) and FP64 only finishes:
+// usually two evaluations, the second with a step below newton_tol. The step's
+// divisor is an FP32 reciprocal (its 1e-7 relative error scales a step that
+// shrinks to nothing, so it moves the number of steps, not the root), and the
+// last step moves sin and cos by their first-order terms (the next is 1e-28).
+// Bracket, safeguard, tolerance and iteration cap are refine_in_cell's: where
+// FP32 does not help (a near-double root, profiles outside FP32's range) the
+// same bisection and Newton steps find the root. With the FP32 sign pass
+// (fp64_signs) it took the FP64 step from 49.2 to 38.6 us at 100 NPs and from 284
+// to 241 us at 2000.
+__device__ __forceinline__ double root_in_cell(const Profile<double> &pf, double S0, double C0,
+                                               float S0f, float C0f, double h, bool left_neg,
+                                               double &s_out, double &c_out) {
+  double x;
+  {
+    const float k2 = static_cast<float>(pf.k2), bc = static_cast<float>(pf.bc),
+                bs = static_cast<float>(pf.bs), hf = static_cast<float>(h);
+    float xf = 0.5f * hf;
+#pragma unroll
+    for (int it = 0; it < 3; ++it) {
+      float sd, cd;
+      Prec<float>::sincos_small(xf, sd, cd);
+      const float s = fmaf(S0f, cd, C0f * sd), c = fmaf(C0f, cd, -S0f * sd);
+      const float d = profile_d1(k2, bc, bs, s, c);
+      const float dd = k2 * (c * c - s * s) + fmaf(bc, c, bs * s);
+      xf = fminf(fmaxf(xf - __fdividef(d, dd), 0.0f), hf);  // (a NaN becomes 0)
+    }
+    x = static_cast<double>(xf);
+  }
+  double lo = 0.0, hi = h;
+  if (!(x > lo && x < hi)) x = 0.5 * h;
+  for (int it = 0; it < Prec<double>::newton_max; ++it) {
+    double sd, cd;
+    Prec<double>::sincos_small(x, sd, cd);
+    const double s = fma(S0, cd, C0 * sd), c = fma(C0, cd, -S0 * sd);
+    const double d = pf.d1(s, c);
+    if (d == 0.0) {
+      s_out = s;
+      c_out = c;
+      return x;
+    }
+    if ((d < 0.0) == left_neg)
+      lo = x;
+    else
+      hi = x;
+    const double dd = pf.d2(s, c);
+    const float ddf = static_cast<float>(dd);
+    const double step = (fabsf(ddf) > 1e-30f && fabsf(ddf) < 1e30f)
+                            ? d * static_cast<double>(__frcp_rn(ddf))
+                            : d / dd;
+    double xn = x - step;
+    if (fabs(step) < Prec<double>::newton_tol) {
+      s_out = fma(-step, c, s);
+      c_out = fma(step, s, c);
+      return xn;
+    }
+    if (!(xn > lo && xn < hi)) xn = 0.5 * (lo + hi);
+    const bool done = hi - lo < Prec<double>::newton_tol;
+    x = xn;
+    if (done) break;
+  }
+  double sd, cd;
+  Prec<double>::sincos_small(x, sd, cd);
+  s_out = fma(S0, cd, C0 * sd);
+  c_out = fma(C0, cd, -S0 * sd);
+  return x;
+}
+
+// FP32 copy of a profile for the FP64 path's sign pass, with the bound on its
+// error. With u = 2^-24, de/dth formed in FP32 from rounded coefficients and
+// table entries errs by at most 6 u (|2k| + |b cos phi| + |b sin phi|) (one
+// rounding each of the coefficient, the sine, the cosine and the operations);
+// guard is 16.8 u times that sum. A value beyond the guard has the FP64 sign;
+// the others are evaluated in FP64. Outside FP32's comfortable range (or not
+// finite) the guard is infinite: every node is evaluated in FP64.
+struct SignProfile {
+  float k2, bc, nbs, guard;
+  __device__ SignProfile(double k2d, double bcd, double bsd) {
+    k2 = static_cast<float>(k2d);
+    bc = static_cast<float>(bcd);
+    nbs = static_cast<float>(-bsd);
+    const float sum = fabsf(k2) + fabsf(bc) + fabsf(nbs);
+    guard = (sum > 1e-25f && sum < 1e30f) ? 1e-6f * sum : INFINITY;
+  }
+};
+
+// Nodes per segment of the scan at most.
+constexpr int kMaxSeg = 50;
+
+// FP32 sign pass over kPairBatch consecutive nodes j0 + q0 .. (j0 + q0 even):
+// two nodes per packed instruction, read as pairs from the split sin and cos
+// tables, each node with profile_d1's roundings (s (2k c + b cos phi) +
+// (-b sin phi) c; a packed operation rounds each half as the scalar one), so
+// the signs are those of the scalar pass. Bit q of the result: node q0 + q.
+constexpr int kPairBatch = 14;
+__device__ __forceinline__ unsigned long long pair_signs(const ScanPairs &tab, f2 K2, f2 BC,
+                                                         f2 NBS, int j0, int q0) {
+  unsigned bits = 0;
+#pragma unroll
+  for (int u = 0; u < kPairBatch; u += 2) {
+    const int j = j0 + q0 + u;  // < kGridPad: the tables repeat the grid past its end
+    const f2 s = *reinterpret_cast<const f2 *>(&tab.ss[j]);
+    const f2 c = *reinterpret_cast<const f2 *>(&tab.cc[j]);
+    const f2 d = fma2(s, fma2(K2, c, BC), mul2(NBS, c));
+    float dl, dh;
+    upk(d, dl, dh);
+    bits |= (static_cast<unsigned>(dl < 0.f) << u) | (static_cast<unsigned>(dh < 0.f) << (u + 1));
+  }
+  return static_cast<unsigned long long>(bits) << q0;
+}
+
+// Signs of the FP64 de/dth at nodes j0 .. j0 + len (bit q: negative at node j0 +
+// q, cyclically; len <= kMaxSeg): the FP32 pass, then FP64 at the nodes whose
+// FP32 value lies within its error bound (SignProfile), so that every bit is
+// that of the FP64 evaluation. Such nodes are rare (a root within about 1e-6 rad
+// of one), and the FP64 pipe, at 1/64 of the FP32 rate, stays free.
+__device__ __forceinline__ unsigned long long fp64_signs(const GridTables<double> &tab,
+                                                         const Profile<double> &pf,
+                                                         const SignProfile &sp, int j0, int len) {
+  const f2 K2 = pk(sp.k2, sp.k2), BC = pk(sp.bc, sp.bc), NBS = pk(sp.nbs, sp.nbs);
+  const int odd = j0 & 1, je = j0 - odd, le = len + odd;  // the packed pairs start on even nodes
+  unsigned long long neg = 0, unsure = 0;
+#pragma unroll 1
+  for (int q0 = 0; q0 <= le; q0 += kPairBatch) {
+    unsigned nb = 0, ub = 0;
+#pragma unroll
+    for (int u = 0; u < kPairBatch; u += 2) {
+      const int j = je + q0 + u;  // < kGridPad: the tables repeat the grid past its end
+      const f2 s = *reinterpret_cast<const f2 *>(&tab.ss[j]);
+      const f2 c = *reinterpret_cast<const f2 *>(&tab.cc[j]);
+      float dl, dh;
+      upk(fma2(s, fma2(K2, c, BC), mul2(NBS, c)), dl, dh);
+      nb |= (static_cast<unsigned>(dl < 0.f) << u) | (static_cast<unsigned>(dh < 0.f) << (u + 1));
+      ub |= (static_cast<unsigned>(!(fabsf(dl) > sp.guard)) << u) |
+            (static_cast<unsigned>(!(fabsf(dh) > sp.guard)) << (u + 1));
+    }
+    neg |= static_cast<unsigned long long>(nb) << q0;
+    unsure |= static_cast<unsigned long long>(ub) << q0;
+  }
+  neg >>= odd;
+  unsure = (unsure >> odd) & ((2ull << len) - 1);
+  while (unsure) {
+    const int q = __ffsll(static_cast<long long>(unsure)) - 1;
+    unsure &= unsure - 1;
+    const int j = j0 + q < kGrid ? j0 + q : j0 + q - kGrid;
+    const bool n = pf.d1(tab.sc[j].x, tab.sc[j].y) < 0.0;
+    neg = (neg & ~(1ull << q)) | (static_cast<unsigned long long>(n) << q);
+  }
+  return neg;
 }
 
 // 1 if x lies on the arc running counter-clockwise from just after `from` up

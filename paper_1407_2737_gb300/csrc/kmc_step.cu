@@ -123,30 +123,6 @@ struct EpiShared {
 // the sign changes (at most four per target) and records each in a free slot of
 // its target (shared-memory counter). All lanes of a warp read the same node,
 // a shared-memory broadcast.
-constexpr int kMaxSeg = 50;
-
-// FP32 sign pass over kPairBatch consecutive nodes j0 + q0 .. (j0 + q0 even):
-// two nodes per packed instruction, read as pairs from the split sin and cos
-// tables, each node with profile_d1's roundings (s (2k c + b cos phi) +
-// (-b sin phi) c; a packed operation rounds each half as the scalar one), so
-// the signs are those of the scalar pass. Bit q of the result: node q0 + q.
-constexpr int kPairBatch = 14;
-__device__ __forceinline__ unsigned long long pair_signs(const GridTables<float> &tab, f2 K2,
-                                                         f2 BC, f2 NBS, int j0, int q0) {
-  unsigned bits = 0;
-#pragma unroll
-  for (int u = 0; u < kPairBatch; u += 2) {
-    const int j = j0 + q0 + u;  // < kGridPad: the tables repeat the grid past its end
-    const f2 s = *reinterpret_cast<const f2 *>(&tab.ss[j]);
-    const f2 c = *reinterpret_cast<const f2 *>(&tab.cc[j]);
-    const f2 d = fma2(s, fma2(K2, c, BC), mul2(NBS, c));
-    float dl, dh;
-    upk(d, dl, dh);
-    bits |= (static_cast<unsigned>(dl < 0.f) << u) | (static_cast<unsigned>(dh < 0.f) << (u + 1));
-  }
-  return static_cast<unsigned long long>(bits) << q0;
-}
-
 template <typename R, bool MULTI = false>
 __device__ __forceinline__ void segment_scan(EpiShared<R> &sm, const GridTables<R> &tab,
                                              int warp, int nw, int lane, int nt) {
@@ -186,13 +162,39 @@ __device__ __forceinline__ void segment_scan(EpiShared<R> &sm, const GridTables<
       }
     }
   };
-  // FP32 segments that start on an even node take the packed pass
+  // FP32 segments that start on an even node take the packed pass; FP64 ones
+  // take their signs from fp64_signs, and keep the sign alone (Newton starts
+  // from an FP32 root)
   constexpr bool kPairs = std::is_same<R, float>::value;
   f2 K2 = 0, BC = 0, NBS = 0;
   if constexpr (kPairs) {
     K2 = pk(k2, k2);
     BC = pk(bc, bc);
     NBS = pk(-bs, -bs);
+  }
+  if constexpr (!kPairs) {
+    static_assert(!MULTI, "FP64 blocks have four warps or more");
+    Profile<double> pf;
+    pf.k2 = k2;
+    pf.k = 0.0;
+    pf.bc = bc;
+    pf.bs = bs;
+    const SignProfile sp(k2, bc, bs);
+    const int seg = (kGrid + nw - 1) / nw;
+    const int j0 = warp * seg, len = min(kGrid, j0 + seg) - j0;
+    if (len <= 0) return;
+    const unsigned long long neg = fp64_signs(tab, pf, sp, j0, len);
+    unsigned long long chg = (neg ^ (neg >> 1)) & ((1ull << len) - 1);
+    while (chg) {
+      const int q = __ffsll(static_cast<long long>(chg)) - 1;
+      chg &= chg - 1;
+      const int slot = atomicAdd(&sm.cnt[lane], 1);
+      if (slot < 4) {
+        sm.ju[lane][slot] = j0 + q;
+        sm.du[lane][slot] = ((neg >> q) & 1) ? -1.0 : 1.0;
+      }
+    }
+    return;
   }
   auto scan = [&](int j0, int len) {
     unsigned long long neg = 0;
@@ -365,7 +367,11 @@ __device__ __forceinline__ void refine_bracket(EpiShared<R> &sm, const GridTable
   const R h = tab.th[1] - tab.th[0];
   R s, c;
   const R dl = sm.du[t][q];
-  const R off = refine_in_cell(pf, sc.x, sc.y, h, dl, sm.duh[t][q], s, c);
+  R off;
+  if constexpr (std::is_same<R, double>::value)
+    off = root_in_cell(pf, sc.x, sc.y, tab.ss[j], tab.cc[j], h, dl < 0.0, s, c);
+  else
+    off = refine_in_cell(pf, sc.x, sc.y, h, dl, sm.duh[t][q], s, c);
   R th = tab.th[j] + off;
   if (th >= Prec<R>::two_pi) th -= Prec<R>::two_pi;
   sm.jq[t][rank] = ju;
