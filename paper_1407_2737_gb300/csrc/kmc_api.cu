@@ -2164,7 +2164,7 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   }
   // device copies, freed on every path out
   struct Buffers {
-    void *p[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    void *p[9] = {};
     cudaStream_t st = nullptr;
     ~Buffers() {
       if (st) cudaStreamSynchronize(st);
@@ -2182,6 +2182,16 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   KMC_TRY(dalloc(reinterpret_cast<double **>(&b.p[4]), sizeof(double) * S));
   KMC_TRY(dalloc(reinterpret_cast<long long **>(&b.p[5]), sizeof(long long) * nl));
   KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&b.p[6]), sizeof(int32_t)));
+  // steps solved at once: as many as 64 MB hold (at least one), the launch's grid
+  // bounding them too
+  const size_t per_step = static_cast<size_t>(N) * (kmc::kMeanFields * sizeof(double) +
+                                                    sizeof(int32_t));
+  const int span = static_cast<int>(std::min<long long>(
+      std::min(S, 65536), std::max<long long>(1, static_cast<long long>((64u << 20) / per_step))));
+  KMC_TRY(dalloc(reinterpret_cast<double **>(&b.p[7]),
+                 sizeof(double) * N * (kmc::kMeanState + kmc::kMeanFields * static_cast<size_t>(span))));
+  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&b.p[8]),
+                 sizeof(int32_t) * N * static_cast<size_t>(span)));
   double *d_bv = static_cast<double *>(b.p[3]);
   KMC_CUDA(cudaMemcpyAsync(b.p[0], hl.data(), sizeof(kmc::MeanLysDev) * n_lys,
                            cudaMemcpyHostToDevice, b.st));
@@ -2208,6 +2218,11 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   a.cos_k = static_cast<const double *>(b.p[4]);
   a.loop = static_cast<long long *>(b.p[5]);
   a.err = static_cast<int32_t *>(b.p[6]);
+  a.n = static_cast<int32_t>(N);
+  a.span = span;
+  a.state = static_cast<double *>(b.p[7]);
+  a.wells = a.state + static_cast<size_t>(N) * kmc::kMeanState;
+  a.flags = static_cast<int32_t *>(b.p[8]);
   KMC_CUDA(kmc::launch_mean(a, b.st));
   std::vector<long long> fx(nl);
   int32_t err = 0;

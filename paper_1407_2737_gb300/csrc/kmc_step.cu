@@ -2395,8 +2395,16 @@ cudaError_t step_blocks_per_sm(int prec_fp32, int warps, int tile, int tpl, int 
 
 cudaError_t launch_mean(const MeanArgs &a, cudaStream_t st) {
   if (a.n_items <= 0) return cudaSuccess;
-  const int blocks = (a.n_items + kMeanWarps - 1) / kMeanWarps;
-  kmc_mean_kernel<<<blocks, kMeanWarps * 32, 0, st>>>(a);
+  for (int p = 0; p < a.periods; ++p)
+    for (int k0 = 0; k0 < a.S; k0 += a.span) {
+      const int k1 = k0 + a.span < a.S ? k0 + a.span : a.S;
+      // a span that holds the whole period serves every period
+      if (p == 0 || a.span < a.S) {
+        const dim3 grid(a.n_items, (k1 - k0 + kMeanWarps - 1) / kMeanWarps);
+        kmc_mean_wells<<<grid, kMeanWarps * 32, 0, st>>>(a, k0, k1);
+      }
+      kmc_mean_carry<<<a.n_items, 32, 0, st>>>(a, k0, k1, p, p == 0 && k0 == 0);
+    }
   return cudaGetLastError();
 }
 

@@ -225,6 +225,19 @@ struct MeanArgs {
   const double *cos_k;   // [S] cos(2 pi k / S)
   long long *loop;       // [n_lys][n_rec] volume-weighted <m_z>, units of 2^-62
   int32_t *err;
+  int32_t n;             // NPs of all lysosomes
+  int32_t span;          // steps per pass of the two kernels (the workspace's)
+  double *wells;         // [span][kMeanFields][n] per (step, NP): angles of the two minima
+                         // and the two maxima, equilibrium occupation of the first
+                         // minimum and the decay towards it, mean m_z of each minimum
+  int32_t *flags;        // [span][n] number of minima | kMean* bits
+  double *state;         // [kMeanState][n] wells' angles, probabilities, mean m_z
+};
+constexpr int kMeanFields = 8, kMeanState = 6;
+enum : int32_t {
+  kMeanArc = 4,    // the first minimum lies on the arc from the first maximum to the second
+  kMeanRelax = 8,  // the occupations relax (T > 0 and a rate above 0)
+  kMeanSkip = 16,  // more than two minima or maxima: the step is skipped, an error set
 };
 
 // Sample regeneration between loops (kmc_regen.cuh), one lysosome per launch.

@@ -1,9 +1,11 @@
 """The FP64 search for the extrema of Eq. 2 (FP32 sign pass with FP64 inside its
-error bound, Newton from an FP32 root) at the places where it can go wrong:
-roots on the nodes of the scan, profiles near switching, a flat or single-term
-profile, magnitudes outside FP32's range.
+error bound, Newton from an FP32 root) and the mean mode's two kernels, at the
+places where they can go wrong: roots on the nodes of the scan, profiles near
+switching, a flat or single-term profile, magnitudes outside FP32's range, and
+runs cut into several spans of steps.
 
-Tolerance: that of the FP64 step (moments 1e-12), a few ulp per operation.
+Tolerances: those of the FP64 step (moments 1e-12) and of the mean mode (1e-12),
+which rest on a few ulp per operation; cut runs are compared bit for bit.
 """
 import math
 
@@ -69,3 +71,24 @@ def test_near_switching(eps):
     for p in (0.2, 0.7, 1.3):
         h = (math.sin(p) ** (2 / 3) + math.cos(p) ** (2 / 3)) ** -1.5
         _check(_lone([math.pi - p], 2e4), h * (1 + eps) * 2 * 2e4 / MS)
+
+
+def test_mean_mode_in_spans():
+    # 10 000 NPs x 200 steps exceed the workspace, so the period is solved in
+    # several spans, anew in each period; the others fit and are solved once
+    big = inputs.lattice_nodes_lysosome(10000, 14e-9, 0.1, Keff=2e4, seed=1)
+    small = inputs.lattice_nodes_lysosome(33, 14e-9, 0.1, Keff=2e4, seed=2)
+    one = _lone([1.0], 2e4, T=0.0)[0]
+    g = kmc.kmc_mean_run([small, big, one], 0.03, 1e5, 200, 2, 0)
+    assert np.array_equal(kmc.kmc_mean_run([small, one], 0.03, 1e5, 200, 2, 0), g[[0, 2]])
+    for q, ly in ((0, small), (2, one)):
+        o = oracle.mean_run(ly.axis, ly.vol, ly.Ms, ly.Keff, ly.T, ly.tau0, 0.03, 1e5, 200, 2, 0)
+        np.testing.assert_allclose(g[q], o, rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("S,H,K", [(1, 0.02, 2e4), (7, 0.0, 2e4), (7, 0.0, 0.0)])
+def test_mean_mode_small(S, H, K):
+    ly = inputs.lattice_nodes_lysosome(3, 14e-9, 0.1, Keff=K, seed=3)
+    g = kmc.kmc_mean_run([ly], H, 1e5, S, 2, 1)
+    o = oracle.mean_run(ly.axis, ly.vol, ly.Ms, ly.Keff, ly.T, ly.tau0, H, 1e5, S, 2, 1)
+    np.testing.assert_allclose(g[0], o, rtol=0, atol=1e-12)
