@@ -151,9 +151,13 @@ struct Shape {
   // 1: the whole field period as one persistent cooperative launch (FP32, one
   // target per lane) with a grid barrier after each step
   int persist = 0;
+  // symmetric form of FP64 contexts, the autotuner's alone: parts per cell pair
+  // (1, 2, 4, 8 or 16; warps = 4, tile = 32, chunk = 0); 0 = the ordered kernel
+  int f64 = 0;
   bool operator==(const Shape &o) const {
     return warps == o.warps && tile == o.tile && chunk == o.chunk && tpl == o.tpl &&
-           rpl == o.rpl && sym == o.sym && cl == o.cl && supd == o.supd && persist == o.persist;
+           rpl == o.rpl && sym == o.sym && cl == o.cl && supd == o.supd && persist == o.persist &&
+           f64 == o.f64;
   }
 };
 
@@ -242,6 +246,15 @@ struct kmc_ctx {
   size_t sfwd_cap = 0, srev_cap = 0;  // floats
   int n_sitems = 0, n_supd = 0;
   std::vector<int> sym_cut_items, sym_cut_upd;
+  // symmetric form in FP64: the same
+  kmc::F64Item *d_fitems = nullptr;
+  size_t fitems_cap = 0;
+  kmc::F64Upd *d_fupd = nullptr;
+  size_t fupd_cap = 0;
+  double *d_f64part = nullptr;
+  size_t f64part_cap = 0;  // doubles
+  int n_fitems = 0, n_fupd = 0;
+  std::vector<int> f64_cut_items, f64_cut_upd;
   int form_mode = 0;           // pair form: 0 = the autotuner's choice, 1 = ordered, 2 = symmetric
   int cl_mode = 0;             // cluster split: 0 = the autotuner's choice, 1 = off, 2 = on
   int supd_mode = 0;           // symmetric update: 0 = the autotuner's, 1 = warp, 2 = block per item
@@ -520,6 +533,71 @@ kmc_status set_sym_items(kmc_ctx *c, const Shape &sh) {
   return KMC_OK;
 }
 
+// Cell pairs of the FP64 symmetric form over all lysosomes.
+long long f64_pairs(const kmc_ctx *c) {
+  long long n = 0;
+  for (int x : c->n) {
+    const long long nc = (x + kmc::kTargets - 1) / kmc::kTargets;
+    n += nc * (nc + 1) / 2;
+  }
+  return n;
+}
+
+// The FP64 symmetric form's plan, `parts` parts per cell pair: lysosomes
+// largest first, each as its cell pairs in order (their parts in order) and one
+// update item per cell; chains cut at lysosome boundaries as in plan_sym.
+kmc_status set_f64_items(kmc_ctx *c, const Shape &sh) {
+  const int parts = sh.f64;
+  int log_parts = 0;
+  while ((1 << log_parts) < parts) ++log_parts;
+  std::vector<int> order(c->n_lys);
+  for (int l = 0; l < c->n_lys; ++l) order[l] = l;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return c->n[x] > c->n[y]; });
+  const int chains = std::min(c->n_lys, kMaxChains);
+  double total = 0.0, acc = 0.0;
+  for (int x : c->n) total += static_cast<double>(x) * x;
+  std::vector<kmc::F64Item> items;
+  std::vector<kmc::F64Upd> upd;
+  std::vector<int> cut_items(1, 0), cut_upd(1, 0);
+  items.reserve(static_cast<size_t>(f64_pairs(c)) * parts);
+  for (int oi = 0; oi < c->n_lys; ++oi) {
+    const int l = order[oi], n = c->n[l], off = c->off[l];
+    const int nc = (n + kmc::kTargets - 1) / kmc::kTargets;
+    const int slot0 = static_cast<int>(items.size());
+    auto cell = [&](int g) { return std::min(kmc::kTargets, n - g * kmc::kTargets); };
+    for (int g = 0; g < nc; ++g) {
+      for (int h = g; h < nc; ++h)
+        for (int p = 0; p < parts; ++p)
+          items.push_back({off + g * kmc::kTargets, off + h * kmc::kTargets, cell(g), cell(h),
+                           32 * p / parts, 32 * (p + 1) / parts, static_cast<int>(items.size()),
+                           0});
+      upd.push_back({l, g * kmc::kTargets, cell(g), g, nc, log_parts, slot0, 0});
+    }
+    acc += static_cast<double>(n) * n;
+    const int q = static_cast<int>(cut_items.size());
+    if (oi + 1 < c->n_lys && q < chains && acc * chains >= total * q) {
+      cut_items.push_back(static_cast<int>(items.size()));
+      cut_upd.push_back(static_cast<int>(upd.size()));
+    }
+  }
+  cut_items.push_back(static_cast<int>(items.size()));
+  cut_upd.push_back(static_cast<int>(upd.size()));
+  KMC_CUDA(cudaStreamSynchronize(c->stream));
+  KMC_TRY(grow(c, &c->d_fitems, &c->fitems_cap, items.size()));
+  KMC_TRY(grow(c, &c->d_fupd, &c->fupd_cap, upd.size()));
+  KMC_TRY(grow(c, &c->d_f64part, &c->f64part_cap, items.size() * kmc::kF64Slot));
+  KMC_CUDA(cudaMemcpy(c->d_fitems, items.data(), sizeof(kmc::F64Item) * items.size(),
+                      cudaMemcpyHostToDevice));
+  KMC_CUDA(cudaMemcpy(c->d_fupd, upd.data(), sizeof(kmc::F64Upd) * upd.size(),
+                      cudaMemcpyHostToDevice));
+  c->n_fitems = static_cast<int>(items.size());
+  c->n_fupd = static_cast<int>(upd.size());
+  c->f64_cut_items = cut_items;
+  c->f64_cut_upd = cut_upd;
+  c->items_shape = sh;
+  return KMC_OK;
+}
+
 template <typename T>
 kmc_status grow(kmc_ctx *c, T **p, size_t *cap, size_t need) {
   if (need <= *cap && *p) return KMC_OK;
@@ -533,11 +611,12 @@ kmc_status grow(kmc_ctx *c, T **p, size_t *cap, size_t need) {
 }
 
 kmc_status set_items(kmc_ctx *c, const Shape &sh) {
-  if (c->items_shape == sh && (sh.sym ? c->d_sitems != nullptr : c->d_items != nullptr))
+  if (c->items_shape == sh && (sh.sym ? c->d_sitems != nullptr
+                                      : sh.f64 ? c->d_fitems != nullptr : c->d_items != nullptr))
     return KMC_OK;
-  if (sh.sym) {
+  if (sh.sym || sh.f64) {
     c->items_shape = Shape();
-    return set_sym_items(c, sh);
+    return sh.sym ? set_sym_items(c, sh) : set_f64_items(c, sh);
   }
   // until the rebuild completes, no shape's items are valid
   c->items_shape = Shape();
@@ -640,6 +719,10 @@ StepArgs base_args(kmc_ctx *c) {
   a.sfwd = c->d_sfwd;
   a.srev = c->d_srev;
   a.n_upd = c->n_supd;
+  a.fitems = c->d_fitems;
+  a.fupd = c->d_fupd;
+  a.f64part = c->d_f64part;
+  a.n_slots = c->n_fitems;
   a.cosk = c->d_cosk;
   a.gbar = c->d_gbar;
   a.barrier_ns = 2000000000ull;  // 2 s
@@ -677,9 +760,10 @@ cudaError_t launch_period(kmc_ctx *c, StepArgs a, const Shape &sh, int steps) {
   return e;
 }
 
-// Chains of the current items (the symmetric form has its own cut).
+// Chains of the current items (the symmetric forms have their own cuts).
 int n_chains_of(const kmc_ctx *c, const Shape &sh) {
-  return static_cast<int>(sh.sym ? c->sym_cut_items.size() : c->chain_cut.size()) - 1;
+  return static_cast<int>(sh.sym ? c->sym_cut_items.size()
+                                 : sh.f64 ? c->f64_cut_items.size() : c->chain_cut.size()) - 1;
 }
 
 // One step of every item of a (all chains, one stream), shape sh.
@@ -692,6 +776,11 @@ cudaError_t launch_one_step(const kmc_ctx *c, StepArgs a, const Shape &sh, cudaS
     a.n_upd = c->n_supd;
     a.gc = sh.warps * sh.sym;
     return kmc::launch_sym(a, sh.warps, sh.sym, c->n_sitems, st, pdl, sh.supd);
+  }
+  if (sh.f64) {
+    a.n_items = c->n_fitems;
+    a.n_upd = c->n_fupd;
+    return kmc::launch_f64sym(a, st, pdl);
   }
   return kmc::launch_step(c->fp32, sh.warps, sh.tile, a, c->n_items, st, pdl, sh.tpl, sh.rpl,
                           sh.cl);
@@ -757,6 +846,9 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
       return false;
     return s.chunk >= 0 && s.chunk % kmc::kCell == 0;
   }
+  if (s.f64 != 0)
+    return !c->fp32 && s.tpl == 1 && s.rpl == 1 && s.cl == 0 && s.warps == 4 && s.tile == 32 &&
+           s.chunk == 0 && s.f64 > 0 && s.f64 <= 16 && (s.f64 & (s.f64 - 1)) == 0;
   if (s.tpl > 3) return false;
   if (s.cl != 0 && (s.cl != 2 || !c->fp32 || s.tpl != 1 || s.rpl != 1 || s.chunk <= 0))
     return false;
@@ -812,6 +904,20 @@ kmc_status capture_steps(kmc_ctx *c, const StepArgs &a, const Shape &sh, int ste
         if (period) b.k_local = k;
         b.cos_k = std::cos(2.0 * kPi * k / steps);
         ce = kmc::launch_sym(b, sh.warps, sh.sym, b.n_items, st, true, sh.supd);
+      }
+      continue;
+    }
+    if (sh.f64) {
+      StepArgs b = a;
+      const int u0 = c->f64_cut_items[q], v0 = c->f64_cut_upd[q];
+      b.fitems = c->d_fitems + u0;
+      b.n_items = c->f64_cut_items[q + 1] - u0;
+      b.fupd = c->d_fupd + v0;
+      b.n_upd = c->f64_cut_upd[q + 1] - v0;
+      for (int k = 0; k < steps && ce == cudaSuccess; ++k) {
+        if (period) b.k_local = k;
+        b.cos_k = std::cos(2.0 * kPi * k / steps);
+        ce = kmc::launch_f64sym(b, st, true);
       }
       continue;
     }
@@ -969,8 +1075,9 @@ kmc_status autotune(kmc_ctx *c) {
     if (!log) return;
     std::fprintf(stderr,
                  "kmc tune %s: warps %d tile %d chunk %d tpl %d rpl %d sym %d cl %d supd %d "
-                 "persist %d: %.4f ms per step\n",
-                 what, s.warps, s.tile, s.chunk, s.tpl, s.rpl, s.sym, s.cl, s.supd, s.persist, ms);
+                 "persist %d f64 %d: %.4f ms per step\n",
+                 what, s.warps, s.tile, s.chunk, s.tpl, s.rpl, s.sym, s.cl, s.supd, s.persist,
+                 s.f64, ms);
   };
   auto consider = [&](const Shape &s, float ms) {
     show("shape", s, ms);
@@ -1036,6 +1143,25 @@ kmc_status autotune(kmc_ctx *c) {
       }
     }
   }
+  // symmetric form in FP64: cell pairs cut in parts while the items are fewer
+  // than the warps that the SMs hold (32 blocks of one warp each, 152 SMs); its
+  // partial sums take 1.5 KB per item, at most 1 GB
+  // (KMC_TUNE_F64=parts, for tests: that many parts, whatever the timings)
+  const char *f64_env = c->fp32 ? nullptr : std::getenv("KMC_TUNE_F64");
+  const int f64_pin = f64_env ? std::atoi(f64_env) : 0;
+  for (int parts = 1; parts <= 16 && !c->fp32 && c->form_mode != 1; parts *= 2) {
+    const long long items = f64_pairs(c) * parts;
+    if (f64_pin > 0) {
+      if (parts != f64_pin) continue;
+    } else if ((parts > 1 && items > 32 * 152) ||
+        items * kmc::kF64Slot * static_cast<long long>(sizeof(double)) > (1ll << 30))
+      break;
+    Shape s;
+    s.warps = 4;
+    s.tile = 32;
+    s.f64 = parts;
+    consider(s, time_shape(c, s));
+  }
   const int warps_c[] = {4, 8};
   const int tiles_f32[] = {64, 128, 256, 512};
   const int tiles_f64[] = {32, 64, 128, 128};  // (the FP64 list has three distinct tiles)
@@ -1062,6 +1188,7 @@ kmc_status autotune(kmc_ctx *c) {
     }
   }
   for (int w : warps_c) {
+    if (f64_pin > 0 && bs.f64 > 0) break;
     if (c->rpl_mode > 1 || sym_only) break;  // pinned replicas or form: only their shapes
     for (int q = 0; q < (c->fp32 ? 4 : 3); ++q) {
       const int t = c->fp32 ? tiles_f32[q] : tiles_f64[q];
@@ -1155,7 +1282,8 @@ void free_ctx(kmc_ctx *c) {
                   c->d_dh,    c->d_pos64,  c->d_phi,     c->d_nodes,    c->d_possi, c->d_phif,
                   c->d_loop,  c->d_cnt,    c->d_err,     c->d_rs,       c->d_items,
                   c->d_partial, c->d_arrivals, c->d_dbg, c->d_dbg_flags, c->d_sitems,
-                  c->d_supd,  c->d_sfwd,   c->d_srev,    c->d_cosk,     c->d_gbar};
+                  c->d_supd,  c->d_sfwd,   c->d_srev,    c->d_cosk,     c->d_gbar,
+                  c->d_fitems, c->d_fupd,  c->d_f64part};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   for (int q = 0; q < kMaxChains; ++q) {
@@ -1544,11 +1672,13 @@ kmc_status kmc_pair_form(kmc_ctx *c, int32_t form, int32_t *form_out) {
       return fail(KMC_EINVAL, "the ordered kernels run 1, 2 or 3 targets per lane");
     c->form_mode = form;
     // a change drops the shape in use: the next run or step tunes, or takes kmc_tuning's
-    if (c->shape.warps != 0 && form != 0 && (c->shape.sym != 0) != (form == 2)) c->shape = Shape();
+    if (c->shape.warps != 0 && form != 0 &&
+        (c->shape.sym != 0 || c->shape.f64 != 0) != (form == 2))
+      c->shape = Shape();
   }
   if (form_out)
     *form_out = c->form_mode != 0 ? c->form_mode
-                                  : (c->shape.warps ? (c->shape.sym ? 2 : 1) : 0);
+                                  : (c->shape.warps ? (c->shape.sym || c->shape.f64 ? 2 : 1) : 0);
   return KMC_OK;
 }
 
@@ -2438,6 +2568,14 @@ kmc_status kmc_debug_stall(kmc_ctx *c) {
   if (c->fp32) return fail(KMC_EINVAL, "the stall hook runs on FP64 contexts");
   KMC_TRY(check_device_error(c));
   KMC_TRY(ensure_shape(c));
+  // the staged copies are the ordered kernel's; the symmetric form has none
+  Shape sh = c->shape;
+  if (sh.f64) {
+    sh = Shape();
+    sh.warps = 4;
+    sh.tile = 64;
+    KMC_TRY(set_items(c, sh));
+  }
   RunState rs{c->step_global, -1, 0};
   KMC_CUDA(cudaMemcpyAsync(c->d_rs, &rs, sizeof(rs), cudaMemcpyHostToDevice, c->stream));
   if (c->arrivals_cap)
@@ -2448,7 +2586,7 @@ kmc_status kmc_debug_stall(kmc_ctx *c) {
   a.cos_k = 1.0;
   a.stall_tx = 16;
   a.stall_wait_ns = 1000000ull;  // 1 ms
-  KMC_CUDA(kmc::launch_step(c->fp32, c->shape.warps, c->shape.tile, a, c->n_items, c->stream));
+  KMC_CUDA(kmc::launch_step(c->fp32, sh.warps, sh.tile, a, c->n_items, c->stream));
   const kmc_status st = check_device_error(c);  // KMC_ETIMEOUT when the waits ran out
   // the blocks stopped before any write: clear the flag, the context stays usable
   KMC_CUDA(cudaMemsetAsync(c->d_err, 0, 2 * sizeof(int32_t), c->stream));

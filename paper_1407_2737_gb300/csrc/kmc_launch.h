@@ -42,6 +42,9 @@ cudaError_t persist_blocks_per_sm(int warps, int tile, int *blocks);
 // (one block per item).
 cudaError_t launch_sym(const StepArgs &a, int warps, int cells, int n_field, cudaStream_t st,
                        bool pdl = false, int upd = 0);
+// One step of the FP64-plain symmetric form: kmc_field_f64 over
+// a.fitems[0 .. a.n_items), then kmc_update_f64 over a.fupd[0 .. a.n_upd).
+cudaError_t launch_f64sym(const StepArgs &a, cudaStream_t st, bool pdl = false);
 size_t sym_smem_bytes(int warps, int cells);
 cudaError_t sym_blocks_per_sm(int warps, int cells, int *blocks);
 

@@ -2162,6 +2162,12 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32)
   grid_launch_dependents();
 }
 
+}  // namespace kmc
+
+#include "kmc_field_f64.cuh"
+
+namespace kmc {
+
 // ---------------------------------------------------------------------------
 // Host side of the launches.
 
@@ -2320,6 +2326,14 @@ cudaError_t launch_sym(const StepArgs &a, int warps, int cells, int n_field, cud
   if (warps == 4 && cells == 2) return launch_sym_wc<4, 2>(a, n_field, st, pdl, upd);
   if (warps == 8 && cells == 1) return launch_sym_wc<8, 1>(a, n_field, st, pdl, upd);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_f64sym(const StepArgs &a, cudaStream_t st, bool pdl) {
+  cudaError_t e = launch_items(kmc_field_f64, a, a.n_items, 32, 0, 0, st, pdl);
+  if (e == cudaSuccess)
+    e = launch_items(kmc_update_f64, a, a.n_upd, kF64UpdWarps * 32,
+                     16 + epi_bytes<double>(kF64UpdWarps), 0, st, pdl);
+  return e;
 }
 
 size_t sym_smem_bytes(int warps, int cells) { return sym_field_smem(warps, cells); }

@@ -127,6 +127,26 @@ __host__ __device__ inline int sym_rev_offset(int h, int gc) {
   return gc * q * (q - 1) / 2 + r * q;
 }
 
+// Symmetric form of the FP64-plain step (kmc_field_f64.cuh): cells of 32 NPs,
+// one warp per pair of cells and range of rotations. Pair (g, h), g <= h, of a
+// lysosome of nc cells has index g nc - g (g - 1) / 2 + h - g; its parts have
+// consecutive slots from the lysosome's first.
+struct F64Item {
+  int32_t g, h;     // first NP of the target and of the source cell (equal: a diagonal pair)
+  int32_t ng, nh;   // their NPs, 1..32
+  int32_t s0, s1;   // rotations [s0, s1) of 32
+  int32_t slot;
+  int32_t pad;
+};
+struct F64Upd {     // one block of kmc_update_f64: a cell's targets
+  int32_t l, t0, nt, cell;
+  int32_t nc;         // cells of the lysosome
+  int32_t log_parts;  // parts per pair, a power of two
+  int32_t slot0;      // the lysosome's first slot
+  int32_t pad;
+};
+constexpr int kF64Slot = 2 * 3 * 32;  // doubles: forward, then reverse sums, [3][32] each
+
 struct RunState {   // advanced on the device at the end of each field period
   long long step_base;  // global index of step 0 of the current period
   int32_t period;       // period index within the run (< 0: not recorded)
@@ -188,6 +208,11 @@ struct StepArgs {
   float *sfwd;
   float *srev;
   int32_t n_upd;
+  // symmetric form in FP64: field items, update items, partial sums [n_slots][kF64Slot]
+  int32_t n_slots;
+  const F64Item *fitems;
+  const F64Upd *fupd;
+  double *f64part;
   // persistent period kernel (kmc_persist_f32): the cosine of each step of the
   // period (host-computed, as the per-step launches receive it), the grid
   // barrier's counters and its time limit; failure-detection test hook: block
