@@ -195,27 +195,66 @@ __device__ __forceinline__ R refine_in_cell(const Profile<R> &pf, R S0, R C0, R 
   return x;
 }
 
+// Start of 1/sqrt(x): the hardware's approximation, whose low word is zero.
+__device__ __forceinline__ double rsqrt_seed(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+
+// 1/sqrt(r2), and 0 for r2 = 0 (a self pair, or two NPs at one point) or an
+// overflowed r2. The seed y has a short mantissa, so y y is exact and e = 1 -
+// r2 y^2 is rounded once; y (1 + e/2 + 3/8 e^2) leaves 5/16 e^3, far below the
+// rounding for a seed good to 2^-20.
+__device__ __forceinline__ double rsqrt_pair(double r2) {
+  const int hi = __double2hiint(r2);
+  const bool none = (hi | __double2loint(r2)) == 0 || hi >= 0x7ff00000;
+  double y = rsqrt_seed(r2);
+  if (none) {
+    y = 0.0;
+    r2 = 0.0;
+  }
+  const double e = fma(-r2, y * y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// sqrt(x) and 1/sqrt(x) to an ulp or two, for x >= 0: a chain of six dependent
+// FP64 operations where sqrt and a division take about thirty. Outside the seed's
+// comfortable range, the functions themselves.
+__device__ __forceinline__ double sqrt_inv(double x, double &inv) {
+  if (x > 1e-290 && x < 1e290) {
+    inv = rsqrt_pair(x);
+    return x * inv;
+  }
+  const double r = sqrt(x);
+  inv = 1.0 / r;
+  return r;
+}
+
 // FP64 root of de/dth inside grid cell [theta_j, theta_j + h] (left_neg: de/dth
 // is negative at theta_j), as offset from theta_j; (S0, C0) = sin, cos of
 // theta_j, (S0f, C0f) the same in FP32. FP64 instructions issue at 1/64 of the
-// FP32 rate here, so the search runs in FP32 until its rounding (about 1e-8
-// rad from the cell's middle in three Newton steps) and FP64 only finishes:
-// usually two evaluations, the second with a step below newton_tol. The step's
-// divisor is an FP32 reciprocal (its 1e-7 relative error scales a step that
-// shrinks to nothing, so it moves the number of steps, not the root), and the
-// last step moves sin and cos by their first-order terms (the next is 1e-28).
-// Bracket, safeguard, tolerance and iteration cap are refine_in_cell's: where
-// FP32 does not help (a near-double root, profiles outside FP32's range) the
-// same bisection and Newton steps find the root. With the FP32 sign pass
-// (fp64_signs) it took the FP64 step from 49.2 to 38.6 us at 100 NPs and from 284
-// to 241 us at 2000.
+// FP32 rate here, and a dependent one takes 60 cycles or so, so the search runs in
+// FP32 until its rounding (about 1e-8 rad from the cell's middle in three Newton
+// steps) and FP64 only finishes, in one evaluation: the step with its second-order
+// term, d = D + C D^2 with D = f / f' and C = f'' / (2 f') (C in FP32: it scales a
+// correction of 1e-15), leaves about C^2 D^3, below 1e-18 under the conditions
+// tested. The divisor is an FP32 reciprocal with one FP64 Newton step (1e-14
+// relative). sin and cos move with the step to second order (the next term is
+// below 2e-19). Where that does not hold (a near-double root, profiles outside
+// FP32's range) the safeguarded Newton iteration of refine_in_cell runs, with its
+// bracket, tolerance and cap. With the FP32 sign pass (fp64_signs) it took the
+// FP64 step from 49.2 to 38.6 us at 100 NPs and from 284 to 241 us at 2000, with
+// two to three evaluations each; one evaluation took the mean mode's wells from
+// 350 to 291 us (2000 NPs x 200 steps).
 __device__ __forceinline__ double root_in_cell(const Profile<double> &pf, double S0, double C0,
                                                float S0f, float C0f, double h, bool left_neg,
                                                double &s_out, double &c_out) {
   double x;
+  const float k2 = static_cast<float>(pf.k2);
   {
-    const float k2 = static_cast<float>(pf.k2), bc = static_cast<float>(pf.bc),
-                bs = static_cast<float>(pf.bs), hf = static_cast<float>(h);
+    const float bc = static_cast<float>(pf.bc), bs = static_cast<float>(pf.bs),
+                hf = static_cast<float>(h);
     float xf = 0.5f * hf;
 #pragma unroll
     for (int it = 0; it < 3; ++it) {
@@ -240,15 +279,25 @@ __device__ __forceinline__ double root_in_cell(const Profile<double> &pf, double
       c_out = c;
       return x;
     }
+    const double dd = pf.d2(s, c);
+    const float ddf = static_cast<float>(dd), df = static_cast<float>(d);
+    const float r = __frcp_rn(ddf), stepf = df * r;
+    // C D, with f'' = -3 (2k) sin cos at the root
+    const float cstep = -1.5f * k2 * static_cast<float>(s) * static_cast<float>(c) * r * stepf;
+    const bool range = fabsf(ddf) > 1e-30f && fabsf(ddf) < 1e30f;
+    if (range && fabsf(stepf) < 1e-6f && fabsf(cstep) < 1e-6f && x > 2e-6 && x < h - 2e-6) {
+      const double rd = static_cast<double>(r);
+      const double step = d * fma(rd, fma(-dd, rd, 1.0), rd);
+      const double full = fma(static_cast<double>(cstep), step, step);
+      s_out = fma(-full, fma(0.5 * full, s, c), s);
+      c_out = fma(full, fma(-0.5 * full, c, s), c);
+      return x - full;
+    }
     if ((d < 0.0) == left_neg)
       lo = x;
     else
       hi = x;
-    const double dd = pf.d2(s, c);
-    const float ddf = static_cast<float>(dd);
-    const double step = (fabsf(ddf) > 1e-30f && fabsf(ddf) < 1e30f)
-                            ? d * static_cast<double>(__frcp_rn(ddf))
-                            : d / dd;
+    const double step = range ? d * static_cast<double>(r) : d / dd;
     double xn = x - step;
     if (fabs(step) < Prec<double>::newton_tol) {
       s_out = fma(-step, c, s);

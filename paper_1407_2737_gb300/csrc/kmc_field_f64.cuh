@@ -21,36 +21,12 @@
 // instructions per ordered pair. Every item writes its sums to its own slot, and
 // the update adds a target's slots in a fixed order: results are deterministic
 // and do not depend on the batch. Per step against the ordered
-// kernel at its best shape: 100 NPs 24.8 against 38.6 us (parts 1, 2, 4, 8, 16:
-// 57.3, 38.7, 29.8, 25.9, 26.1), 400: 32 against 65, 1000: 61 against 98, 2000: 160
-// against 239, 4000: 528 against 772, where the pipe is 87 % busy. The autotuner
-// times both.
+// kernel at its best shape: 100 NPs 18.5 against 36 us (parts 2, 4, 8, 16: 35.1,
+// 25.7, 21.2, 20.4), 400: 26 against 62, 1000: 54 against 73, 2000: 152 against 214,
+// 4000: 523 against 754, where the pipe is 88 % busy. The autotuner times both.
 #pragma once
 
 namespace kmc {
-
-// Start of 1/sqrt(x): the hardware's approximation, whose low word is zero.
-__device__ __forceinline__ double rsqrt_seed(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-
-// 1/sqrt(r2), and 0 for r2 = 0 (a self pair, or two NPs at one point) or an
-// overflowed r2. The seed y has a short mantissa, so y y is exact and e = 1 -
-// r2 y^2 is rounded once; y (1 + e/2 + 3/8 e^2) leaves 5/16 e^3, far below the
-// rounding for a seed good to 2^-20.
-__device__ __forceinline__ double rsqrt_pair(double r2) {
-  const int hi = __double2hiint(r2);
-  const bool none = (hi | __double2loint(r2)) == 0 || hi >= 0x7ff00000;
-  double y = rsqrt_seed(r2);
-  if (none) {
-    y = 0.0;
-    r2 = 0.0;
-  }
-  const double e = fma(-r2, y * y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
 
 struct F64Src {  // position and 3 w m of one NP (n = -w m is t times -1/3: kept apart)
   double x, y, z, tx, ty, tz, nx, ny, nz;
@@ -101,9 +77,14 @@ __global__ void __launch_bounds__(32) kmc_field_f64(const StepArgs a, int /*tile
   double fx = 0.0, fy = 0.0, fz = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
   const int from = (lane + 1) & 31;
   auto move = [&](double v) { return __shfl_sync(0xffffffffu, v, from); };
+  auto next = [&](const F64Src &v) {
+    return F64Src{move(v.x),  move(v.y),  move(v.z),  move(v.tx), move(v.ty),
+                  move(v.tz), move(v.nx), move(v.ny), move(v.nz)};
+  };
   if (diag) {
 #pragma unroll 2
     for (int r = s0; r < it.s1; ++r) {
+      const F64Src ahead = next(s);  // independent of this rotation's sums
       const double dx = s.x - t.x, dy = s.y - t.y, dz = s.z - t.z;
       const double q = rsqrt_pair(fma(dx, dx, fma(dy, dy, dz * dz)));
       const double q2 = q * q, q3 = q * q2;
@@ -111,19 +92,12 @@ __global__ void __launch_bounds__(32) kmc_field_f64(const StepArgs a, int /*tile
       fx = fma(q3, fma(u, dx, s.nx), fx);
       fy = fma(q3, fma(u, dy, s.ny), fy);
       fz = fma(q3, fma(u, dz, s.nz), fz);
-      s.x = move(s.x);
-      s.y = move(s.y);
-      s.z = move(s.z);
-      s.tx = move(s.tx);
-      s.ty = move(s.ty);
-      s.tz = move(s.tz);
-      s.nx = move(s.nx);
-      s.ny = move(s.ny);
-      s.nz = move(s.nz);
+      s = ahead;
     }
   } else {
 #pragma unroll 2
     for (int r = s0; r < it.s1; ++r) {
+      const F64Src ahead = next(s);  // independent of this rotation's sums
       const double dx = s.x - t.x, dy = s.y - t.y, dz = s.z - t.z;
       const double q = rsqrt_pair(fma(dx, dx, fma(dy, dy, dz * dz)));
       const double q2 = q * q, q3 = q * q2;
@@ -136,15 +110,7 @@ __global__ void __launch_bounds__(32) kmc_field_f64(const StepArgs a, int /*tile
       rx = move(fma(q3, fma(v, dx, t.nx), rx));
       ry = move(fma(q3, fma(v, dy, t.ny), ry));
       rz = move(fma(q3, fma(v, dz, t.nz), rz));
-      s.x = move(s.x);
-      s.y = move(s.y);
-      s.z = move(s.z);
-      s.tx = move(s.tx);
-      s.ty = move(s.ty);
-      s.tz = move(s.tz);
-      s.nx = move(s.nx);
-      s.ny = move(s.ny);
-      s.nz = move(s.nz);
+      s = ahead;
     }
   }
   // the slot: forward sums [3][32] by target, reverse sums [3][32] by source
@@ -207,7 +173,8 @@ __global__ void __launch_bounds__(kF64UpdWarps * 32)
            (p < c ? 96 : 0) + lane;
   };
   double h0 = 0.0, h1 = 0.0, h2 = 0.0;
-  constexpr int kBatch = 4;  // slots whose loads are issued before any is added
+  constexpr int kBatch = 8;  // slots loaded together and added pairwise: a chain of
+                             // three dependent additions and one instead of eight
 #pragma unroll 1
   for (int x0 = warp; x0 < total; x0 += NW * kBatch) {
     double v[kBatch][3];
@@ -216,15 +183,17 @@ __global__ void __launch_bounds__(kF64UpdWarps * 32)
       const bool in = x0 + b * NW < total;
       const double *p = sums(in ? x0 + b * NW : x0);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) v[b][q] = __ldcg(p + 32 * q);
+      for (int q = 0; q < 3; ++q) v[b][q] = in ? __ldcg(p + 32 * q) : 0.0;
     }
 #pragma unroll
-    for (int b = 0; b < kBatch; ++b) {
-      if (x0 + b * NW >= total) break;
-      h0 += v[b][0];
-      h1 += v[b][1];
-      h2 += v[b][2];
-    }
+    for (int w = 1; w < kBatch; w *= 2)
+#pragma unroll
+      for (int b = 0; b < kBatch; b += 2 * w)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[b][q] += v[b + w][q];
+    h0 += v[0][0];
+    h1 += v[0][1];
+    h2 += v[0][2];
   }
   double *wp = reinterpret_cast<double *>(dyn);  // [NW][3][32]
   wp[(warp * 3 + 0) * 32 + lane] = h0;

@@ -399,21 +399,33 @@ __device__ __forceinline__ TargetState<R> setup_plane(R ax, R ay, R az, R mx, R 
   s.ay = ay;
   s.az = az;
   s.mz_old = mz;
-  s.bmag = sqrt(fma(bx, bx, fma(by, by, bz * bz)));
+  // FP64: the square roots and divisions of the usual branch by sqrt_inv
+  constexpr bool kFast = std::is_same<R, double>::value;
+  const R b2 = fma(bx, bx, fma(by, by, bz * bz));
+  R binv = R(0);
+  if constexpr (kFast)
+    s.bmag = sqrt_inv(b2, binv);
+  else
+    s.bmag = sqrt(b2);
   s.ex = s.ey = s.ez = R(0);
   s.cphi = R(1);
   s.sphi = R(0);
   s.degenerate = true;
   if (s.bmag > R(0)) {
-    const R inv = R(1) / s.bmag;
+    const R inv = kFast ? binv : R(1) / s.bmag;
     const R hx = bx * inv, hy = by * inv, hz = bz * inv;
     R cphi = fma(ax, hx, fma(ay, hy, az * hz));
     const R px = fma(-cphi, ax, hx), py = fma(-cphi, ay, hy), pz = fma(-cphi, az, hz);
-    const R sp = sqrt(fma(px, px, fma(py, py, pz * pz)));
+    const R sp2 = fma(px, px, fma(py, py, pz * pz));
+    R sinv = R(0), sp;
+    if constexpr (kFast)
+      sp = sqrt_inv(sp2, sinv);
+    else
+      sp = sqrt(sp2);
     if (sp >= Prec<R>::plane_tol) {
-      s.ex = px / sp;
-      s.ey = py / sp;
-      s.ez = pz / sp;
+      s.ex = kFast ? px * sinv : px / sp;
+      s.ey = kFast ? py * sinv : py / sp;
+      s.ez = kFast ? pz * sinv : pz / sp;
       s.sphi = sp;
       s.degenerate = false;
     } else {
@@ -443,10 +455,34 @@ __device__ __forceinline__ TargetState<R> setup_plane(R ax, R ay, R az, R mx, R 
   }
   s.m_a = fma(mx, ax, fma(my, ay, mz * az));
   s.m_e = fma(mx, s.ex, fma(my, s.ey, mz * s.ez));
-  R th0 = atan2(s.m_e, s.m_a);
-  if (th0 < R(0)) th0 += Prec<R>::two_pi;
-  s.th0 = th0;
+  if constexpr (kFast) {  // FP32: decide takes the FP64 angle where this one is too near
+    float th0 = atan2f(static_cast<float>(s.m_e), static_cast<float>(s.m_a));
+    if (th0 < 0.0f) th0 += Prec<float>::two_pi;
+    s.th0 = th0;
+  } else {
+    R th0 = atan2(s.m_e, s.m_a);
+    if (th0 < R(0)) th0 += Prec<R>::two_pi;
+    s.th0 = th0;
+  }
   return s;
+}
+
+// Whether the projected moment lies on the arc from M1 to M2 (step v). FP64: the
+// FP32 angle decides (its error and the rounding of M1 and M2 to FP32 are below
+// 2e-6 rad) unless it lies within 1e-5 rad of either end.
+__device__ __forceinline__ bool moment_on_arc(const TargetState<float> &st, float M1, float M2) {
+  return on_arc<float>(st.th0, M1, M2);
+}
+__device__ __forceinline__ bool moment_on_arc(const TargetState<double> &st, double M1,
+                                              double M2) {
+  const float t = static_cast<float>(st.th0), m1 = static_cast<float>(M1),
+              m2 = static_cast<float>(M2);
+  const float d1 = fabsf(t - m1), d2 = fabsf(t - m2);
+  const float near = fminf(fminf(d1, Prec<float>::two_pi - d1), fminf(d2, Prec<float>::two_pi - d2));
+  if (near > 1e-5f) return on_arc<float>(t, m1, m2);
+  double th0 = atan2(st.m_e, st.m_a);
+  if (th0 < 0.0) th0 += Prec<double>::two_pi;
+  return on_arc<double>(th0, M1, M2);
 }
 
 struct Decision {
@@ -466,12 +502,17 @@ __device__ __forceinline__ float exp_fp64_arg(double x) {
 
 // Steps v-vii for target t: basins, barrier (FP64 polish near the switching
 // field in the mixed path), Eqs. 3-5 in FP64, draw u < P. Returns (sin, cos)
-// of the new angle in the plane.
+// of the new angle in the plane. FP64 path: unless exact_p asks for P itself (the
+// debug outputs), FP32 exponentials of the FP64 exponents settle u < P wherever u
+// lies further from that P than its error and the near-threshold band (1e-9)
+// together; otherwise P is formed in FP64. The decision is the FP64 one either
+// way; its two exponentials, expm1 and division are some 90 dependent FP64
+// operations of about 60 cycles each.
 template <typename R, bool MIXED>
 __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
                                            const TargetState<R> &st, double beta,
-                                           double lognu0t, bool t_zero, double u, R &s_new,
-                                           R &c_new) {
+                                           double lognu0t, bool t_zero, double u, bool exact_p,
+                                           R &s_new, R &c_new) {
   Decision o;
   o.dEa = o.dEb = o.P = 0.0;
   o.flipped = o.near = o.bad = o.polished = 0;
@@ -508,7 +549,7 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
   }
   // v) basins: the two maxima split the circle into two arcs
   const R M1 = sm.th[t][imax0], M2 = sm.th[t][imax1];
-  const bool arc0 = on_arc<R>(st.th0, M1, M2);
+  const bool arc0 = moment_on_arc(st, M1, M2);
   const bool arcA = on_arc<R>(sm.th[t][imin0], M1, M2);
   const int wa = (arc0 == arcA) ? imin0 : imin1;
   const int wb = (wa == imin0) ? imin1 : imin0;
@@ -553,10 +594,22 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
       const float sum = ea + eb;
       P = (sum > 0.f) ? static_cast<double>((ea / sum) * (-expm1f(-sum))) : 0.0;
     } else {
-      const double ea = exp(lognu0t - beta * dEa);
-      const double eb = exp(lognu0t - beta * dEb);
-      const double sum = ea + eb;
-      P = (sum > 0.0) ? (ea / sum) * (-expm1(-sum)) : 0.0;
+      const double xa = lognu0t - beta * dEa, xb = lognu0t - beta * dEb;
+      bool settled = false;
+      P = 0.0;
+      if (!exact_p) {
+        // relative error of Pf below 1.2e-6: 2 ulp in each exponential, then
+        // the sum, the quotient, expm1 and the product; a NaN (overflow) is not settled
+        const float ea = exp_fp64_arg(xa), eb = exp_fp64_arg(xb), sum = ea + eb;
+        const float Pf = (sum > 0.f) ? (ea / sum) * (-expm1f(-sum)) : 0.f;
+        const float uf = static_cast<float>(u);
+        settled = fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
+        P = Pf;
+      }
+      if (!settled) {
+        const double ea = exp(xa), eb = exp(xb), sum = ea + eb;
+        P = (sum > 0.0) ? (ea / sum) * (-expm1(-sum)) : 0.0;
+      }
     }
     o.P = P;
     // vii) jump iff u < P
@@ -709,7 +762,7 @@ __device__ __forceinline__ void block_update(
   // lanes past the last target repeat the last target (same state as st);
   // only targets < nt have scan results in shared memory
   const Decision r = decide<R, MIXED>(sm, min(lane, nt - 1), st, tin.beta, L.lognu0t,
-                                      L.t_zero != 0, u, s_new, c_new);
+                                      L.t_zero != 0, u, a.debug != 0, s_new, c_new);
   // Guard: a non-finite field, barrier or probability (two NPs at one point)
   // leaves the moment as it was; the NP-step is counted and reported.
   const bool finite = isfinite(sm.h[0][lane]) && isfinite(sm.h[1][lane]) &&
