@@ -28,8 +28,8 @@
 // the nodes within its error (SignProfile) and Newton starts from an FP32 root
 // (root_in_cell). 2000 NPs, 200 steps: 75.4 ms with one
 // thread per NP for the whole run (63 warps on 152 SMs, every step a serial chain
-// of about 1.7e4 FP64 instructions), 0.97 ms now, of which the wells take 0.35 ms
-// and the carry 0.24 ms.
+// of about 1.7e4 FP64 instructions), 0.85 ms now, of which the wells take 0.29 ms
+// and the carry 0.18 ms.
 #pragma once
 
 namespace kmc {
@@ -173,89 +173,125 @@ __global__ void __launch_bounds__(kMeanWarps * 32)
   }
 }
 
-// One warp per item: the probabilities through steps k0 .. k1 - 1 of period p,
-// from and to the state of the NPs (a.state; first: the start of the run).
-__global__ void __launch_bounds__(32)
+// One block per item of 32 NPs: the probabilities through steps k0 .. k1 - 1 of
+// period p, from and to the state of the NPs (a.state; first: the start of the
+// run), in tiles of kCarryTile steps. Warp 0 runs the chain of a tile, which is
+// all that is serial (occupations of a step from those before it); meanwhile the
+// other warps load the next tile's wells into shared memory and reduce the
+// previous tile's contributions to the loop. One warp doing all three took 242 us
+// for 200 steps of 2000 NPs. Now 180 us.
+constexpr int kCarryTile = 8, kCarryHelpers = 4;
+
+__global__ void __launch_bounds__(32 * (1 + kCarryHelpers))
     kmc_mean_carry(const MeanArgs a, int k0, int k1, int p, int first) {
-  const int lane = threadIdx.x;
+  __shared__ double s_well[2][kCarryTile][kMeanFields][32];
+  __shared__ double s_mz[2][kCarryTile][32];
+  __shared__ int s_flag[2][kCarryTile][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const MeanItem it = a.items[blockIdx.x];
   const MeanLysDev L = a.lys[it.l];
   const bool active = lane < it.nt;
   const int i = L.off + it.t0 + min(lane, it.nt - 1);
-  const double vfrac = active ? a.vfrac[i] : 0.0;
-  // the wells as of the last step that had any: angles, probabilities (0 for a
-  // well that does not exist) and mean m_z
-  double th0, th1, p0, p1, g0, g1;
-  double *st = a.state + i;
-  if (first) {  // all probability in the well along +-a with m_z >= 0
-    th0 = (a.axis[i].z >= 0.0) ? 0.0 : 0.5 * Prec<double>::two_pi;
-    th1 = 0.0;
-    p0 = 1.0;
-    p1 = 0.0;
-    g0 = fabs(a.axis[i].z);
-    g1 = 0.0;
-  } else {
-    th0 = st[0];
-    th1 = st[a.n];
-    p0 = st[2ll * a.n];
-    p1 = st[3ll * a.n];
-    g0 = st[4ll * a.n];
-    g1 = st[5ll * a.n];
-  }
-  bool bad = false;
-  struct Wells {
-    double v[kMeanFields];
-    int flag;
-  };
-  auto load = [&](int k) {
-    Wells w;
-    const double *src = a.wells + static_cast<size_t>(k - k0) * kMeanFields * a.n + i;
+  const int steps = k1 - k0, tiles = (steps + kCarryTile - 1) / kCarryTile;
+  // helpers: the wells of tile t, the steps in turn
+  auto load = [&](int t) {
+    for (int q = warp - 1; q < kCarryTile; q += kCarryHelpers) {
+      const int r = t * kCarryTile + q;
+      if (r >= steps) break;
+      const double *src = a.wells + static_cast<size_t>(r) * kMeanFields * a.n + i;
+      double v[kMeanFields];
 #pragma unroll
-    for (int f = 0; f < kMeanFields; ++f) w.v[f] = src[static_cast<size_t>(f) * a.n];
-    w.flag = a.flags[static_cast<size_t>(k - k0) * a.n + i];
-    return w;
+      for (int f = 0; f < kMeanFields; ++f) v[f] = src[static_cast<size_t>(f) * a.n];
+      const int flag = a.flags[static_cast<size_t>(r) * a.n + i];
+#pragma unroll
+      for (int f = 0; f < kMeanFields; ++f) s_well[t & 1][q][f][lane] = v[f];
+      s_flag[t & 1][q][lane] = flag;
+    }
   };
-  Wells next = load(k0);
-  for (int k = k0; k < k1; ++k) {
-    const Wells w = next;
-    if (k + 1 < k1) next = load(k + 1);  // ahead of this step's chain
-    const int nmin = w.flag & 3;
-    const bool skip = (w.flag & kMeanSkip) != 0;
-    bad = bad || (active && skip);
-    if (nmin == 1) {
-      p0 = 1.0;
-      p1 = 0.0;
-    } else if (nmin == 2) {
-      const double M1 = w.v[2], M2 = w.v[3];
-      const bool arcA = (w.flag & kMeanArc) != 0;
-      const bool in0 = on_arc<double>(th0, M1, M2) == arcA;
-      const bool in1 = on_arc<double>(th1, M1, M2) == arcA;
-      double pA = (in0 ? p0 : 0.0) + (in1 ? p1 : 0.0);
-      double pB = (in0 ? 0.0 : p0) + (in1 ? 0.0 : p1);
-      if (w.flag & kMeanRelax) {
-        pA = w.v[4] + (pA - w.v[4]) * w.v[5];
-        pB = 1.0 - pA;
-      }
-      p0 = pA;
-      p1 = pB;
-    }
-    if (nmin != 0 && !skip) {
-      th0 = w.v[0];
-      th1 = w.v[1];
-      g0 = w.v[6];
-      g1 = w.v[7];
-    }
-    if (p >= a.discard) {
-      double c = skip ? 0.0 : vfrac * (p0 * g0 + p1 * g1);
+  // helpers: the volume-weighted sums of tile t into the loop record
+  auto reduce = [&](int t) {
+    if (p < a.discard) return;
+    for (int q = warp - 1; q < kCarryTile; q += kCarryHelpers) {
+      const int r = t * kCarryTile + q;
+      if (r >= steps) break;
+      double c = s_mz[t & 1][q][lane];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
       if (lane == 0) {
-        const long long rec = static_cast<long long>(p - a.discard) * a.S + k;
+        const long long rec = static_cast<long long>(p - a.discard) * a.S + k0 + r;
         atomicAdd(reinterpret_cast<unsigned long long *>(
                       &a.loop[static_cast<long long>(it.l) * a.n_rec + rec]),
                   static_cast<unsigned long long>(__double2ll_rn(c * kLoopScale)));
       }
     }
+  };
+  // warp 0: the wells as of the last step that had any: angles, probabilities (0
+  // for a well that does not exist) and mean m_z
+  double th0 = 0.0, th1 = 0.0, p0 = 1.0, p1 = 0.0, g0 = 0.0, g1 = 0.0, vfrac = 0.0;
+  double *st = a.state + i;
+  bool bad = false;
+  if (warp == 0) {
+    vfrac = active ? a.vfrac[i] : 0.0;
+    if (first) {  // all probability in the well along +-a with m_z >= 0
+      const double az = a.axis[i].z;
+      th0 = (az >= 0.0) ? 0.0 : 0.5 * Prec<double>::two_pi;
+      g0 = fabs(az);
+    } else {
+      th0 = st[0];
+      th1 = st[a.n];
+      p0 = st[2ll * a.n];
+      p1 = st[3ll * a.n];
+      g0 = st[4ll * a.n];
+      g1 = st[5ll * a.n];
+    }
+  } else {
+    load(0);
+  }
+  __syncthreads();
+  for (int t = 0; t < tiles; ++t) {
+    if (warp == 0) {
+      const int cnt = min(kCarryTile, steps - t * kCarryTile);
+#pragma unroll 2
+      for (int q = 0; q < cnt; ++q) {
+        const double(&w)[kMeanFields][32] = s_well[t & 1][q];
+        const int flag = s_flag[t & 1][q][lane];
+        const int nmin = flag & 3;
+        const bool skip = (flag & kMeanSkip) != 0;
+        bad = bad || (active && skip);
+        if (nmin == 1) {
+          p0 = 1.0;
+          p1 = 0.0;
+        } else if (nmin == 2) {
+          const double M1 = w[2][lane], M2 = w[3][lane], pinf = w[4][lane];
+          const bool arcA = (flag & kMeanArc) != 0;
+          const bool in0 = on_arc<double>(th0, M1, M2) == arcA;
+          const bool in1 = on_arc<double>(th1, M1, M2) == arcA;
+          double pA = (in0 ? p0 : 0.0) + (in1 ? p1 : 0.0);
+          double pB = (in0 ? 0.0 : p0) + (in1 ? 0.0 : p1);
+          if (flag & kMeanRelax) {
+            pA = pinf + (pA - pinf) * w[5][lane];
+            pB = 1.0 - pA;
+          }
+          p0 = pA;
+          p1 = pB;
+        }
+        if (nmin != 0 && !skip) {
+          th0 = w[0][lane];
+          th1 = w[1][lane];
+          g0 = w[6][lane];
+          g1 = w[7][lane];
+        }
+        s_mz[t & 1][q][lane] = skip ? 0.0 : vfrac * (p0 * g0 + p1 * g1);
+      }
+    } else {
+      if (t > 0) reduce(t - 1);
+      if (t + 1 < tiles) load(t + 1);
+    }
+    __syncthreads();
+  }
+  if (warp != 0) {
+    if (tiles > 0) reduce(tiles - 1);
+    return;
   }
   if (active) {
     st[0] = th0;

@@ -2470,7 +2470,7 @@ cudaError_t launch_mean(const MeanArgs &a, cudaStream_t st) {
         const dim3 grid(a.n_items, (k1 - k0 + kMeanWarps - 1) / kMeanWarps);
         kmc_mean_wells<<<grid, kMeanWarps * 32, 0, st>>>(a, k0, k1);
       }
-      kmc_mean_carry<<<a.n_items, 32, 0, st>>>(a, k0, k1, p, p == 0 && k0 == 0);
+      kmc_mean_carry<<<a.n_items, 32 * (1 + kCarryHelpers), 0, st>>>(a, k0, k1, p, p == 0 && k0 == 0);
     }
   return cudaGetLastError();
 }
