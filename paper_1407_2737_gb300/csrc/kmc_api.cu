@@ -217,6 +217,7 @@ struct kmc_ctx {
   void *d_pos64 = nullptr;    // FP32 contexts: [N] dbl4 positions in FP64 (x, y, z, w)
   double *d_phi = nullptr;    // [max n] scratch of kmc_local_concentration
   float4 *d_phif = nullptr;   // [max n] its FP32 copy of the positions
+  void *d_phigrid = nullptr;  // its grid (largest lysosome)
   std::vector<double> len;    // [n_lys] length unit L, m
   std::vector<double> ctr;    // [n_lys][3] frame origin, m
   std::vector<double> pos_si; // [N][3] current positions, m
@@ -1280,6 +1281,7 @@ void free_ctx(kmc_ctx *c) {
   void *ptrs[] = {c->d_lys,   c->d_pos,    c->d_axis,    c->d_m,        c->d_src[0],
                   c->d_src[1], c->d_slot,  c->d_beta,    c->d_vfrac,    c->d_eacc,
                   c->d_dh,    c->d_pos64,  c->d_phi,     c->d_nodes,    c->d_possi, c->d_phif,
+                  c->d_phigrid,
                   c->d_loop,  c->d_cnt,    c->d_err,     c->d_rs,       c->d_items,
                   c->d_partial, c->d_arrivals, c->d_dbg, c->d_dbg_flags, c->d_sitems,
                   c->d_supd,  c->d_sfwd,   c->d_srev,    c->d_cosk,     c->d_gbar,
@@ -2164,17 +2166,33 @@ kmc_status kmc_local_concentration(kmc_ctx *c, int32_t lys, int32_t N, double *p
     KMC_TRY(dalloc(&c->d_phif, sizeof(float4) * max_n));
   }
   const dbl4 *pos = static_cast<const dbl4 *>(c->fp32 ? c->d_pos64 : c->d_pos) + c->off[lys];
-  // largest distance from the frame origin, in units of L (with a little
-  // slack for the rounding of the device's frame coordinates)
-  double rmax = 0.0;
+  if (!c->d_phigrid) {
+    size_t need = 0;
+    for (int x : c->n) need = std::max(need, kmc::local_concentration_scratch(x));
+    if (need) KMC_TRY(dalloc(reinterpret_cast<char **>(&c->d_phigrid), need));
+  }
+  // the box of the positions about the frame origin and their largest distance
+  // from it, in units of L (with a little slack for the rounding of the device's
+  // frame coordinates)
+  double lo[3], hi[3], r2max = 0.0;
+  for (int q = 0; q < 3; ++q) lo[q] = hi[q] = c->pos_si[3ull * c->off[lys] + q] - c->ctr[3 * lys + q];
   for (int i = 0; i < n; ++i) {
     const double *q = &c->pos_si[3ull * (c->off[lys] + i)];
-    const double dx = q[0] - c->ctr[3 * lys], dy = q[1] - c->ctr[3 * lys + 1],
-                 dz = q[2] - c->ctr[3 * lys + 2];
-    rmax = std::max(rmax, std::sqrt(dx * dx + dy * dy + dz * dz));
+    const double d[3] = {q[0] - c->ctr[3 * lys], q[1] - c->ctr[3 * lys + 1],
+                         q[2] - c->ctr[3 * lys + 2]};
+    r2max = std::max(r2max, d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+    for (int k = 0; k < 3; ++k) {
+      lo[k] = std::min(lo[k], d[k]);
+      hi[k] = std::max(hi[k], d[k]);
+    }
   }
-  rmax = 1.01 * rmax / c->len[lys];
-  KMC_CUDA(kmc::launch_local_concentration(pos, n, N, rmax, c->d_phif, c->d_phi, c->stream));
+  const double rmax = 1.01 * std::sqrt(r2max) / c->len[lys];
+  for (int k = 0; k < 3; ++k) {
+    lo[k] /= c->len[lys];
+    hi[k] /= c->len[lys];
+  }
+  KMC_CUDA(kmc::launch_local_concentration(pos, n, N, rmax, lo, hi, c->d_phif, c->d_phigrid,
+                                           c->d_phi, c->stream));
   KMC_CUDA(cudaMemcpyAsync(phi, c->d_phi, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
   KMC_CUDA(cudaStreamSynchronize(c->stream));
   return KMC_OK;
