@@ -148,6 +148,9 @@ struct Shape {
   int cl = 0;
   // symmetric form's update kernel: 0 = one warp per update item, 1 = one block
   int supd = 0;
+  // symmetric form, the autotuner's alone: items of about equal work, bal waves of
+  // the blocks that the SMs hold (chunk = 0); 0 = items of `chunk` source NPs
+  int bal = 0;
   // 1: the whole field period as one persistent cooperative launch (FP32, one
   // target per lane) with a grid barrier after each step
   int persist = 0;
@@ -157,7 +160,7 @@ struct Shape {
   bool operator==(const Shape &o) const {
     return warps == o.warps && tile == o.tile && chunk == o.chunk && tpl == o.tpl &&
            rpl == o.rpl && sym == o.sym && cl == o.cl && supd == o.supd && persist == o.persist &&
-           f64 == o.f64;
+           f64 == o.f64 && bal == o.bal;
   }
 };
 
@@ -241,6 +244,8 @@ struct kmc_ctx {
   // symmetric form: field and update items, their chains, the partial sums
   kmc::SymItem *d_sitems = nullptr;
   size_t sitems_cap = 0;
+  int32_t *d_rslot = nullptr;
+  size_t rslot_cap = 0;
   kmc::SymUpd *d_supd = nullptr;
   size_t supd_cap = 0;
   float *d_sfwd = nullptr, *d_srev = nullptr;
@@ -437,49 +442,114 @@ Plan plan_items(const std::vector<int> &np, bool fp32, int chunk, int blocks_per
 // update lists at the same lysosomes.
 struct SymPlan {
   std::vector<kmc::SymItem> items;
+  std::vector<int> rbase;    // per item, the lysosome's first reverse slot (kmc_plan_sym)
+  std::vector<int> rslot;    // reverse slot per off-diagonal item and source cell
   std::vector<kmc::SymUpd> upd;
   std::vector<int> cut_items, cut_upd;
   long long n_rev = 0;  // reverse slots (forward slots: one per item)
 };
 
-SymPlan plan_sym(const std::vector<int> &np, int gc, int src_cells) {
+// The order of the lysosomes in a plan: largest first, stable.
+std::vector<int> plan_order(const std::vector<int> &np) {
+  std::vector<int> order(np.size());
+  for (size_t l = 0; l < np.size(); ++l) order[l] = static_cast<int>(l);
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return np[x] > np[y]; });
+  return order;
+}
+
+// Equal shares of a row group's work, for items of at most `most` work units: per
+// source cell (kCellRec rotations) a block of the symmetric loop issues 28
+// packed instructions per rotation and target of a lane, one of the ordered loop 18.
+constexpr double kSymCellWork = 28.0, kDiagCellWork = 18.0;
+int shares(double work, double most) { return std::max(1, static_cast<int>(std::ceil(work / most))); }
+
+// Blocks of a batch when no item exceeds `most`: the diagonal and the off-diagonal
+// part of every row group in shares of their own.
+long long balanced_items(const std::vector<int> &np, int gc, double most) {
+  long long n = 0;
+  for (int x : np) {
+    const int nc = (x + kmc::kCell - 1) / kmc::kCell;
+    for (int g = 0; g * gc < nc; ++g) {
+      n += shares(kDiagCellWork * std::min(gc, nc - g * gc), most);
+      if (nc > (g + 1) * gc) n += shares(kSymCellWork * (nc - (g + 1) * gc), most);
+    }
+  }
+  return n;
+}
+
+// max_items = 0: items of src_cells source cells (0: a whole row). max_items > 0:
+// balanced items, at most that many (but one per part of a row group at least),
+// each a run of rotations that may start and end inside a cell. A launch whose
+// items are all resident at once ends with its longest one, and with items cut at
+// whole cells only a lysosome of some thousand NPs has either too few of them
+// for the SMs or items of very different length.
+SymPlan plan_sym(const std::vector<int> &np, int gc, int src_cells, long long max_items = 0) {
   SymPlan p;
   const int n_lys = static_cast<int>(np.size());
-  std::vector<int> order(n_lys);
-  for (int l = 0; l < n_lys; ++l) order[l] = l;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return np[x] > np[y]; });
+  const std::vector<int> order = plan_order(np);
   const int chains = std::min(n_lys, kMaxChains);
   double total = 0.0, acc = 0.0;
   for (int l = 0; l < n_lys; ++l) total += static_cast<double>(np[l]) * np[l];
+  double most = 0.0;
+  if (max_items > 0) {  // the smallest bound on an item's work that the count allows
+    double lo = kDiagCellWork / kmc::kCellRec, hi = kSymCellWork * (1 << 25);
+    for (int k = 0; k < 60; ++k) {
+      const double mid = std::sqrt(lo * hi);
+      (balanced_items(np, gc, mid) <= max_items ? hi : lo) = mid;
+    }
+    most = hi;
+  }
   p.cut_items.assign(1, 0);
   p.cut_upd.assign(1, 0);
   for (int oi = 0; oi < n_lys; ++oi) {
     const int l = order[oi], n = np[l];
     const int nc = (n + kmc::kCell - 1) / kmc::kCell, ng = (nc + gc - 1) / gc;
     const int rbase = static_cast<int>(p.n_rev);
-    p.n_rev += kmc::sym_rev_offset(nc, gc);
-    std::vector<int> g0(ng), gn(ng);
-    for (int g = 0; g < ng; ++g) {
-      g0[g] = static_cast<int>(p.items.size());
-      kmc::SymItem d{};
-      d.l = l;
-      d.g = g;
-      d.h0 = d.h1 = -1;
-      d.fwd = g0[g];
-      d.rbase = rbase;
-      p.items.push_back(d);
-      const int step = src_cells > 0 ? src_cells : nc;
-      for (int h0 = (g + 1) * gc; h0 < nc; h0 += step) {
+    std::vector<int> g0(ng), gn(ng), parts(nc, 0);  // parts: reverse slots of a cell
+    const size_t first = p.items.size();
+    // source cells [c0, c1) of row group g in q items of about equal rotations
+    auto cut = [&](int g, int c0, int c1, int q, bool off) {
+      const long long rot = static_cast<long long>(c1 - c0) * kmc::kCellRec;
+      q = static_cast<int>(std::min<long long>(q, rot / 2));
+      for (int k = 0; k < q; ++k) {
+        const long long a = rot * k / q / 2 * 2, b = k + 1 == q ? rot : rot * (k + 1) / q / 2 * 2;
         kmc::SymItem it{};
         it.l = l;
         it.g = g;
-        it.h0 = h0;
-        it.h1 = std::min(nc, h0 + step);
+        it.h0 = c0 + static_cast<int>(a / kmc::kCellRec);
+        it.h1 = c0 + static_cast<int>((b + kmc::kCellRec - 1) / kmc::kCellRec);
+        it.s0 = static_cast<int>(a % kmc::kCellRec);
+        it.s1 = static_cast<int>((b - 1) % kmc::kCellRec) + 1;
         it.fwd = static_cast<int>(p.items.size());
-        it.rbase = rbase;
+        if (off)
+          for (int h = it.h0; h < it.h1; ++h) ++parts[h];
         p.items.push_back(it);
+        p.rbase.push_back(rbase);
+      }
+    };
+    for (int g = 0; g < ng; ++g) {
+      g0[g] = static_cast<int>(p.items.size());
+      const int c1 = std::min(nc, (g + 1) * gc);
+      cut(g, g * gc, c1, most > 0 ? shares(kDiagCellWork * (c1 - g * gc), most) : 1, false);
+      if (most > 0) {
+        if (c1 < nc) cut(g, c1, nc, shares(kSymCellWork * (nc - c1), most), true);
+      } else {
+        const int step = src_cells > 0 ? src_cells : nc;
+        for (int h0 = c1; h0 < nc; h0 += step) cut(g, h0, std::min(nc, h0 + step), 1, true);
       }
       gn[g] = static_cast<int>(p.items.size()) - g0[g];
+    }
+    // reverse slots: cell by cell, within a cell by row group and then part
+    std::vector<int> rev0(nc), next(nc);
+    for (int h = 0; h < nc; ++h) {
+      rev0[h] = next[h] = static_cast<int>(p.n_rev);
+      p.n_rev += parts[h];
+    }
+    for (size_t u = first; u < p.items.size(); ++u) {
+      kmc::SymItem &it = p.items[u];
+      it.rs0 = static_cast<int>(p.rslot.size());
+      if (it.h0 < (it.g + 1) * gc) continue;
+      for (int h = it.h0; h < it.h1; ++h) p.rslot.push_back(next[h]++);
     }
     for (int t0 = 0; t0 < n; t0 += kmc::kTargets) {
       const int h = t0 / kmc::kCell, g = h / gc;
@@ -489,8 +559,8 @@ SymPlan plan_sym(const std::vector<int> &np, int gc, int src_cells) {
       u.nt = std::min(kmc::kTargets, n - t0);
       u.fwd0 = g0[g];
       u.nfwd = gn[g];
-      u.rev0 = rbase + kmc::sym_rev_offset(h, gc);
-      u.nrev = h / gc;
+      u.rev0 = rev0[h];
+      u.nrev = parts[h];
       u.gt0 = t0 - g * gc * kmc::kCell;
       p.upd.push_back(u);
     }
@@ -514,8 +584,20 @@ kmc_status grow(kmc_ctx *c, T **p, size_t *cap, size_t need);
 kmc_status set_sym_items(kmc_ctx *c, const Shape &sh) {
   const int gc = sh.warps * sh.sym;
   std::vector<int> np(c->n.begin(), c->n.end());
-  const SymPlan plan = plan_sym(np, gc, sh.chunk / kmc::kCell);
+  long long max_items = 0;
+  if (sh.bal > 0) {
+    int dev = 0, n_sms = 0, per_sm = 0;
+    KMC_CUDA(cudaGetDevice(&dev));
+    KMC_CUDA(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
+    KMC_CUDA(kmc::sym_blocks_per_sm(sh.warps, sh.sym, &per_sm));
+    max_items = static_cast<long long>(sh.bal) * per_sm * n_sms;
+  }
+  const SymPlan plan = plan_sym(np, gc, sh.chunk / kmc::kCell, max_items);
   KMC_CUDA(cudaStreamSynchronize(c->stream));
+  KMC_TRY(grow(c, &c->d_rslot, &c->rslot_cap, std::max<size_t>(1, plan.rslot.size())));
+  if (!plan.rslot.empty())
+    KMC_CUDA(cudaMemcpy(c->d_rslot, plan.rslot.data(), sizeof(int32_t) * plan.rslot.size(),
+                        cudaMemcpyHostToDevice));
   KMC_TRY(grow(c, &c->d_sitems, &c->sitems_cap, plan.items.size()));
   KMC_TRY(grow(c, &c->d_supd, &c->supd_cap, plan.upd.size()));
   KMC_TRY(grow(c, &c->d_sfwd, &c->sfwd_cap,
@@ -717,6 +799,7 @@ StepArgs base_args(kmc_ctx *c) {
   }
   a.sitems = c->d_sitems;
   a.supd = c->d_supd;
+  a.rslot = c->d_rslot;
   a.sfwd = c->d_sfwd;
   a.srev = c->d_srev;
   a.n_upd = c->n_supd;
@@ -776,7 +859,7 @@ cudaError_t launch_one_step(const kmc_ctx *c, StepArgs a, const Shape &sh, cudaS
     a.n_items = c->n_sitems;
     a.n_upd = c->n_supd;
     a.gc = sh.warps * sh.sym;
-    return kmc::launch_sym(a, sh.warps, sh.sym, c->n_sitems, st, pdl, sh.supd);
+    return kmc::launch_sym(a, sh.warps, sh.sym, c->n_sitems, st, pdl, sh.supd, sh.bal > 0);
   }
   if (sh.f64) {
     a.n_items = c->n_fitems;
@@ -845,8 +928,10 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
     if (!((s.warps == 4 && (s.sym == 1 || s.sym == 2)) || (s.warps == 8 && s.sym == 1) ||
           (s.warps == 2 && s.sym == 2)))
       return false;
+    if (s.bal < 0 || (s.bal > 0 && s.chunk != 0)) return false;
     return s.chunk >= 0 && s.chunk % kmc::kCell == 0;
   }
+  if (s.bal != 0) return false;
   if (s.f64 != 0)
     return !c->fp32 && s.tpl == 1 && s.rpl == 1 && s.cl == 0 && s.warps == 4 && s.tile == 32 &&
            s.chunk == 0 && s.f64 > 0 && s.f64 <= 16 && (s.f64 & (s.f64 - 1)) == 0;
@@ -904,7 +989,7 @@ kmc_status capture_steps(kmc_ctx *c, const StepArgs &a, const Shape &sh, int ste
       for (int k = 0; k < steps && ce == cudaSuccess; ++k) {
         if (period) b.k_local = k;
         b.cos_k = std::cos(2.0 * kPi * k / steps);
-        ce = kmc::launch_sym(b, sh.warps, sh.sym, b.n_items, st, true, sh.supd);
+        ce = kmc::launch_sym(b, sh.warps, sh.sym, b.n_items, st, true, sh.supd, sh.bal > 0);
       }
       continue;
     }
@@ -1076,9 +1161,9 @@ kmc_status autotune(kmc_ctx *c) {
     if (!log) return;
     std::fprintf(stderr,
                  "kmc tune %s: warps %d tile %d chunk %d tpl %d rpl %d sym %d cl %d supd %d "
-                 "persist %d f64 %d: %.4f ms per step\n",
+                 "persist %d f64 %d bal %d: %.4f ms per step\n",
                  what, s.warps, s.tile, s.chunk, s.tpl, s.rpl, s.sym, s.cl, s.supd, s.persist,
-                 s.f64, ms);
+                 s.f64, s.bal, ms);
   };
   auto consider = [&](const Shape &s, float ms) {
     show("shape", s, ms);
@@ -1106,6 +1191,7 @@ kmc_status autotune(kmc_ctx *c) {
     bs.tpl = 2 * bs.sym;
   }
   // symmetric form (FP32): (warps, cells per warp), source NPs per field item
+  const char *bal_env = std::getenv("KMC_TUNE_BAL");
   if (c->fp32 && c->form_mode != 1 && c->rpl_mode <= 1 &&
       (c->tpl_mode == 0 || c->tpl_mode == 2 || c->tpl_mode == 4)) {
     const int wc[4][2] = {{2, 2}, {4, 1}, {4, 2}, {8, 1}};
@@ -1113,6 +1199,7 @@ kmc_status autotune(kmc_ctx *c) {
       if (c->tpl_mode != 0 && 2 * v[1] != c->tpl_mode) continue;
       const int gc = v[0] * v[1];
       for (int ch : {0, 256, 512, 1024, 2048, 4096}) {
+        if (bal_env) break;
         // a field item of ch source NPs, at least one row group's worth
         if (ch > 0 && (ch >= max_n || ch < gc * kmc::kCell / 2)) continue;
         Shape s;
@@ -1125,13 +1212,29 @@ kmc_status autotune(kmc_ctx *c) {
         const float ms = time_shape(c, s);
         consider(s, ms);
       }
+      // balanced items, 1, 2, 4 or 8 waves of them (tests: KMC_TUNE_BAL, only these)
+      for (int bal : {1, 2, 4, 8}) {
+        if (bal_env && bal != std::atoi(bal_env)) continue;
+        Shape s;
+        s.warps = v[0];
+        s.tile = 32;
+        s.tpl = 2 * v[1];
+        s.sym = v[1];
+        s.bal = bal;
+        // (their targets gather more slots, so both update kernels are timed)
+        for (int supd = 0; supd <= 1; ++supd) {
+          if (c->supd_mode != 0 && c->supd_mode != 1 + supd) continue;
+          s.supd = supd;
+          consider(s, time_shape(c, s));
+        }
+      }
     }
     // the symmetric shapes within 3 % of the best with the other update kernel
     // (shapes that tie with one update kernel can part with the other)
     if (bs.sym && c->supd_mode == 0) {
       std::vector<std::pair<float, Shape>> near;
       for (const auto &t : timed)
-        if (t.second.sym && t.first <= 1.03f * best) near.push_back(t);
+        if (t.second.sym && t.second.bal == 0 && t.first <= 1.03f * best) near.push_back(t);
       std::sort(near.begin(), near.end(),
                 [](const std::pair<float, Shape> &x, const std::pair<float, Shape> &y) {
                   return x.first < y.first;
@@ -1285,7 +1388,7 @@ void free_ctx(kmc_ctx *c) {
                   c->d_loop,  c->d_cnt,    c->d_err,     c->d_rs,       c->d_items,
                   c->d_partial, c->d_arrivals, c->d_dbg, c->d_dbg_flags, c->d_sitems,
                   c->d_supd,  c->d_sfwd,   c->d_srev,    c->d_cosk,     c->d_gbar,
-                  c->d_fitems, c->d_fupd,  c->d_f64part};
+                  c->d_fitems, c->d_fupd,  c->d_f64part, c->d_rslot};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   for (int q = 0; q < kMaxChains; ++q) {
@@ -1573,7 +1676,9 @@ kmc_status kmc_plan_sym(const int32_t *n, int32_t n_lys, int32_t gc, int32_t src
                 (long long)*n_upd);
   for (size_t u = 0; u < p.items.size(); ++u) {
     const kmc::SymItem &it = p.items[u];
-    const int32_t row[KMC_SYM_FIELDS] = {it.l, it.g, it.h0, it.h1, it.fwd, it.rbase, 0, 0};
+    const bool diag = it.h0 < (it.g + 1) * gc;
+    const int32_t row[KMC_SYM_FIELDS] = {it.l,   it.g,       diag ? -1 : it.h0, diag ? -1 : it.h1,
+                                         it.fwd, p.rbase[u], 0,                 0};
     std::memcpy(items_out + KMC_SYM_FIELDS * u, row, sizeof(row));
   }
   for (size_t u = 0; u < p.upd.size(); ++u) {

@@ -39,9 +39,9 @@ cudaError_t persist_blocks_per_sm(int warps, int tile, int *blocks);
 // (warps, cells) in {(2, 2), (4, 1), (4, 2), (8, 1)}; row groups of warps x cells
 // cells (4 or 8).
 // upd: 0 = kmc_update_sym (one warp per update item), 1 = kmc_update_sym_block
-// (one block per item).
+// (one block per item). part: items may start and end inside a cell.
 cudaError_t launch_sym(const StepArgs &a, int warps, int cells, int n_field, cudaStream_t st,
-                       bool pdl = false, int upd = 0);
+                       bool pdl = false, int upd = 0, bool part = false);
 // One step of the FP64-plain symmetric form: kmc_field_f64 over
 // a.fitems[0 .. a.n_items), then kmc_update_f64 over a.fupd[0 .. a.n_upd).
 cudaError_t launch_f64sym(const StepArgs &a, cudaStream_t st, bool pdl = false);

@@ -1814,10 +1814,10 @@ __device__ __forceinline__ void sym_cell(const ulonglong2 *__restrict__ sp, int 
                                          const f2 (&X)[T], const f2 (&Y)[T], const f2 (&Z)[T],
                                          const f2 (&TX)[T], const f2 (&TY)[T], const f2 (&TZ)[T],
                                          const f2 (&NX)[T], const f2 (&NY)[T], const f2 (&NZ)[T],
-                                         AccF32 (&acc)[T], f2 &rx, f2 &ry, f2 &rz) {
+                                         AccF32 (&acc)[T], f2 &rx, f2 &ry, f2 &rz, int s0, int s1) {
   const int from = (lane + 1) & (kCellRec - 1);
 #pragma unroll 2
-  for (int s = 0; s < kCellRec; ++s) {
+  for (int s = s0; s < s1; ++s) {
     ulonglong2 a, b, c, d;
     f2 e;
     load_record(sp, (lane + s) & (kCellRec - 1), a, b, c, d, e);
@@ -1850,9 +1850,9 @@ __device__ __forceinline__ void sym_cell(const ulonglong2 *__restrict__ sp, int 
 template <bool MASK, int T>
 __device__ __forceinline__ void ordered_cell(const ulonglong2 *__restrict__ sp, const f2 (&X)[T],
                                              const f2 (&Y)[T], const f2 (&Z)[T],
-                                             AccF32 (&acc)[T]) {
+                                             AccF32 (&acc)[T], int r0, int r1) {
 #pragma unroll 1
-  for (int r = 0; r < kCellRec; ++r) {
+  for (int r = r0; r < r1; ++r) {
     ulonglong2 a, b, c, d;
     f2 e;
     load_record(sp, r, a, b, c, d, e);
@@ -1869,11 +1869,14 @@ __device__ __forceinline__ bool sym_item_in_bounds(const StepArgs &a, int gc) {
   const SymItem it = a.sitems[blockIdx.x];
   if (!KMC_DCHECK(it.l >= 0 && it.l < a.n_lys, a.err, kSiteLys)) return false;
   const int nc = (a.lys[it.l].n + kCell - 1) / kCell;
-  if (!KMC_DCHECK(it.g >= 0 && it.g * gc < nc && it.fwd >= 0 && it.rbase >= 0, a.err,
+  if (!KMC_DCHECK(it.g >= 0 && it.g * gc < nc && it.fwd >= 0 && it.rs0 >= 0, a.err,
                   kSiteTargets))
     return false;
-  if (!KMC_DCHECK((it.h0 == -1 && it.h1 == -1) ||
-                      (it.h0 >= (it.g + 1) * gc && it.h0 < it.h1 && it.h1 <= nc),
+  const int end = (it.g + 1) * gc;  // the group's cells end here
+  if (!KMC_DCHECK(it.h0 < it.h1 && it.h1 <= nc &&
+                      (it.h0 >= end || (it.h0 >= it.g * gc && it.h1 <= end)) && it.s0 >= 0 &&
+                      it.s0 < kCellRec && it.s1 > 0 && it.s1 <= kCellRec &&
+                      (it.h1 - it.h0 > 1 || it.s0 < it.s1),
                   a.err, kSiteSources))
     return false;
 #endif
@@ -1906,7 +1909,10 @@ constexpr size_t sym_field_smem(int w, int c) {
                    : static_cast<size_t>(w) * c * kCellRec * sizeof(SrcPair));
 }
 
-template <int W, int C>
+// PART: items may start and end inside a cell (balanced plans). Whole cells keep
+// the loops' trip counts constants: with variable ones the whole-cell shapes ran
+// 3-4 % slower (50 000 NPs 1.222 -> 1.263 ms per step, a batch 231 -> 241 us).
+template <int W, int C, bool PART>
 __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*tile*/) {
   constexpr int T = 2 * C;    // targets per lane
   constexpr int GC = W * C;   // cells per row group
@@ -1969,10 +1975,13 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
   };
   ulonglong2 *buf = reinterpret_cast<ulonglong2 *>(dyn);
 
-  if (it.h0 < 0) {
-    // diagonal item: the group's records in one copy, ordered pairs
-    const int c0 = it.g * GC, ncv = min(GC, nc - c0);
-    const uint32_t bytes = static_cast<uint32_t>(ncv) * kCellRec * sizeof(SrcPair);
+  const int ncs = it.h1 - it.h0;
+  // rotations (records) of the item's t-th source cell
+  auto first_of = [&](int t) { return PART && t == 0 ? it.s0 : 0; };
+  auto end_of = [&](int t) { return PART && t == ncs - 1 ? it.s1 : kCellRec; };
+  if (it.h0 < (it.g + 1) * GC) {
+    // diagonal item: its source cells' records in one copy, ordered pairs
+    const uint32_t bytes = static_cast<uint32_t>(ncs) * kCellRec * sizeof(SrcPair);
     if (threadIdx.x == 0) {
       mbar_init(&bar[0], 1);
       mbar_init_fence();
@@ -1980,7 +1989,7 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
     __syncthreads();
     if (threadIdx.x == 0) {
       mbar_expect_tx(&bar[0], bytes);
-      bulk_g2s(buf, gsrc + c0 * kCellRec, bytes, &bar[0]);
+      bulk_g2s(buf, gsrc + it.h0 * kCellRec, bytes, &bar[0]);
     }
     const bool ok = mbar_wait_bounded(&bar[0], 0, a.err);
     if (!__syncthreads_and(ok)) {
@@ -1989,15 +1998,15 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
       return;
     }
 #pragma unroll 1
-    for (int cs = 0; cs < ncv; ++cs) {
+    for (int cs = 0; cs < ncs; ++cs) {
       AccF32 acc[T];
 #pragma unroll
       for (int k = 0; k < T; ++k) acc[k].x = acc[k].y = acc[k].z = 0ull;
       const ulonglong2 *sp = buf + static_cast<size_t>(cs) * kCellRec * kRecU2;
-      if (cs >= warp * C && cs < warp * C + C)
-        ordered_cell<true, T>(sp, X, Y, Z, acc);
+      if (it.h0 + cs >= cell0 && it.h0 + cs < cell0 + C)
+        ordered_cell<true, T>(sp, X, Y, Z, acc, first_of(cs), end_of(cs));
       else
-        ordered_cell<false, T>(sp, X, Y, Z, acc);
+        ordered_cell<false, T>(sp, X, Y, Z, acc, first_of(cs), end_of(cs));
       fold(acc);
     }
   } else {
@@ -2010,11 +2019,10 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
                bytes, &bar[b]);
     };
     // the warps' reverse sums of cell h0 + t, added in warp order into its
-    // slot for this row group: [3][64], component-major
+    // slot for this item: [3][64], component-major
     auto flush_rev = [&](int t) {
       const float *rb = red + (t & 1) * W * 6 * 32;
-      float *dst = a.srev + static_cast<size_t>(it.rbase + sym_rev_offset(it.h0 + t, GC) + it.g) *
-                                3 * kCell;
+      float *dst = a.srev + static_cast<size_t>(a.rslot[it.rs0 + t]) * 3 * kCell;
       for (int v = threadIdx.x; v < 6 * 32; v += W * 32) {
         const int j = v >> 5, ln = v & 31;
         float r = rb[j * 32 + ln];
@@ -2030,21 +2038,21 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
       for (int k = 0; k < T; ++k) acc[k].x = acc[k].y = acc[k].z = 0ull;
       f2 rx = 0ull, ry = 0ull, rz = 0ull;
       sym_cell<T>(buf + static_cast<size_t>(b) * kCellRec * kRecU2, lane, X, Y, Z, TX, TY, TZ, NX,
-                  NY, NZ, acc, rx, ry, rz);
+                  NY, NZ, acc, rx, ry, rz, first_of(t), end_of(t));
       fold(acc);
-      float *rw = red + ((t & 1) * W + warp) * 6 * 32;
+      // the lane now carries the record that its next rotation would have met
+      float *rw = red + ((t & 1) * W + warp) * 6 * 32 + ((lane + end_of(t)) & (kCellRec - 1));
       float lo, hi;
       upk(rx, lo, hi);
-      rw[0 * 32 + lane] = lo;
-      rw[3 * 32 + lane] = hi;
+      rw[0 * 32] = lo;
+      rw[3 * 32] = hi;
       upk(ry, lo, hi);
-      rw[1 * 32 + lane] = lo;
-      rw[4 * 32 + lane] = hi;
+      rw[1 * 32] = lo;
+      rw[4 * 32] = hi;
       upk(rz, lo, hi);
-      rw[2 * 32 + lane] = lo;
-      rw[5 * 32 + lane] = hi;
+      rw[2 * 32] = lo;
+      rw[5 * 32] = hi;
     };
-    const int ncs = it.h1 - it.h0;
     if (!staged_loop(ncs, bar, a.err, issue, body)) return;
     flush_rev(ncs - 1);
   }
@@ -2355,10 +2363,14 @@ cudaError_t launch_persist(const StepArgs &a, int warps, int tile, int n_items, 
 // over the a.n_upd target groups, both on st.
 template <int W, int C>
 static cudaError_t launch_sym_wc(const StepArgs &a, int n_field, cudaStream_t st, bool pdl,
-                                 int upd) {
+                                 int upd, bool part) {
   cudaError_t e = cudaSuccess;
-  if (n_field > 0)
-    e = launch_items(kmc_field_sym<W, C>, a, n_field, W * 32, sym_field_smem(W, C), 0, st, pdl);
+  if (n_field > 0 && part)
+    e = launch_items(kmc_field_sym<W, C, true>, a, n_field, W * 32, sym_field_smem(W, C), 0, st,
+                     pdl);
+  else if (n_field > 0)
+    e = launch_items(kmc_field_sym<W, C, false>, a, n_field, W * 32, sym_field_smem(W, C), 0, st,
+                     pdl);
   if (e == cudaSuccess && a.n_upd > 0) {
     if (upd == 1)
       e = launch_items(kmc_update_sym_block<W * C>, a, a.n_upd, kSymUpdWarps * 32,
@@ -2372,12 +2384,12 @@ static cudaError_t launch_sym_wc(const StepArgs &a, int n_field, cudaStream_t st
 }
 
 cudaError_t launch_sym(const StepArgs &a, int warps, int cells, int n_field, cudaStream_t st,
-                       bool pdl, int upd) {
+                       bool pdl, int upd, bool part) {
   if (upd != 0 && upd != 1) return cudaErrorInvalidValue;
-  if (warps == 2 && cells == 2) return launch_sym_wc<2, 2>(a, n_field, st, pdl, upd);
-  if (warps == 4 && cells == 1) return launch_sym_wc<4, 1>(a, n_field, st, pdl, upd);
-  if (warps == 4 && cells == 2) return launch_sym_wc<4, 2>(a, n_field, st, pdl, upd);
-  if (warps == 8 && cells == 1) return launch_sym_wc<8, 1>(a, n_field, st, pdl, upd);
+  if (warps == 2 && cells == 2) return launch_sym_wc<2, 2>(a, n_field, st, pdl, upd, part);
+  if (warps == 4 && cells == 1) return launch_sym_wc<4, 1>(a, n_field, st, pdl, upd, part);
+  if (warps == 4 && cells == 2) return launch_sym_wc<4, 2>(a, n_field, st, pdl, upd, part);
+  if (warps == 8 && cells == 1) return launch_sym_wc<8, 1>(a, n_field, st, pdl, upd, part);
   return cudaErrorInvalidValue;
 }
 
@@ -2407,10 +2419,10 @@ cudaError_t persist_blocks_per_sm(int warps, int tile, int *blocks) {
 cudaError_t sym_blocks_per_sm(int warps, int cells, int *blocks) {
   *blocks = 0;
   const size_t smem = sym_field_smem(warps, cells);
-  if (warps == 2 && cells == 2) return occupancy(kmc_field_sym<2, 2>, 64, smem, blocks);
-  if (warps == 4 && cells == 1) return occupancy(kmc_field_sym<4, 1>, 128, smem, blocks);
-  if (warps == 4 && cells == 2) return occupancy(kmc_field_sym<4, 2>, 128, smem, blocks);
-  if (warps == 8 && cells == 1) return occupancy(kmc_field_sym<8, 1>, 256, smem, blocks);
+  if (warps == 2 && cells == 2) return occupancy(kmc_field_sym<2, 2, true>, 64, smem, blocks);
+  if (warps == 4 && cells == 1) return occupancy(kmc_field_sym<4, 1, true>, 128, smem, blocks);
+  if (warps == 4 && cells == 2) return occupancy(kmc_field_sym<4, 2, true>, 128, smem, blocks);
+  if (warps == 8 && cells == 1) return occupancy(kmc_field_sym<8, 1, true>, 256, smem, blocks);
   return cudaErrorInvalidValue;
 }
 
@@ -2545,10 +2557,14 @@ cudaError_t init_device() {
   if (e == cudaSuccess) e = allow_smem(kmc_step_f32_rep<4, 2>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f32_rep<2, 4>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f32_rep<4, 4>);
-  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<2, 2>);
-  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 1>);
-  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 2>);
-  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<8, 1>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<2, 2, false>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<2, 2, true>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 1, false>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 1, true>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 2, false>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<4, 2, true>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<8, 1, false>);
+  if (e == cudaSuccess) e = allow_smem(kmc_field_sym<8, 1, true>);
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym<4>);
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym<8>);
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym_block<4>);

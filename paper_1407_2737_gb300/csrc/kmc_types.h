@@ -107,25 +107,21 @@ constexpr int kCellRec = kCell / 2;
 struct SymItem {   // one block of kmc_field_sym
   int32_t l;       // lysosome
   int32_t g;       // row group: target cells g gc .. g gc + gc - 1
-  int32_t h0, h1;  // source cells [h0, h1); h0 = h1 = -1: the group's diagonal item
+  int32_t h0, h1;  // source cells [h0, h1), above the group, or inside it (a diagonal
+                   // item: ordered pairs of the group's targets with those cells)
   int32_t fwd;     // forward-partial slot of this item
-  int32_t rbase;   // first reverse slot of the lysosome
-  int32_t pad[2];
+  int32_t rs0;     // its source cells' reverse slots: rslot[rs0 + h - h0] (off-diagonal)
+  int32_t s0, s1;  // rotations (diagonal: source records) from s0 of cell h0 to s1 of
+                   // cell h1 - 1, of 32 each: an item may start and end inside a cell
 };
 
 struct SymUpd {    // one block of kmc_update_sym: up to 32 targets of one cell
   int32_t l, t0, nt;    // lysosome, first target, targets (1..32)
   int32_t fwd0, nfwd;   // forward-partial slots of the target's row group (consecutive)
-  int32_t rev0, nrev;   // reverse slots of the targets' cell, one per row group below
+  int32_t rev0, nrev;   // reverse slots of the targets' cell (consecutive), one per
+                        // item of a row group below that holds rotations of the cell
   int32_t gt0;          // t0 minus the first target of the row group
 };
-
-// First reverse slot of cell h within its lysosome: cell h' holds one slot
-// per row group below it, floor(h' / gc) of them.
-__host__ __device__ inline int sym_rev_offset(int h, int gc) {
-  const int q = h / gc, r = h % gc;
-  return gc * q * (q - 1) / 2 + r * q;
-}
 
 // Symmetric form of the FP64-plain step (kmc_field_f64.cuh): cells of 32 NPs,
 // one warp per pair of cells and range of rotations. Pair (g, h), g <= h, of a
@@ -205,6 +201,7 @@ struct StepArgs {
   // components per target of the row group), reverse [slot][3][64]
   const SymItem *sitems;
   const SymUpd *supd;
+  const int32_t *rslot;
   float *sfwd;
   float *srev;
   int32_t n_upd;
