@@ -304,6 +304,24 @@ kmc_status dalloc(T **p, size_t bytes) {
   return KMC_OK;
 }
 
+// Device scratch of one call: its arrays are added up in a first pass, taken from
+// one allocation in a second, and freed with it on every return.
+struct Scratch {
+  char *p = nullptr;
+  size_t used = 0;
+  Scratch() = default;
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
+  ~Scratch() {
+    if (p) cudaFree(p);
+  }
+  template <typename T>
+  void take(T **out, size_t count) {
+    if (p) *out = reinterpret_cast<T *>(p + used);
+    used += (sizeof(T) * count + 255) / 256 * 256;
+  }
+};
+
 void drop_graph(kmc_ctx *c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   c->gexec = nullptr;
@@ -2509,25 +2527,8 @@ kmc_status kmc_regenerate_rsa(kmc_ctx *c, int32_t lys, double radius, double dia
     KMC_CUDA(cudaMemcpy(c->d_possi, c->pos_si.data(), sizeof(double) * 3 * c->N,
                         cudaMemcpyHostToDevice));
   }
-  // scratch, freed on every return
   const int B = static_cast<int>(
       std::min<long long>(kmc::kRsaMaxBatch, std::max<long long>(256, 2ll * n)));
-  struct Scratch {
-    void *p[8] = {};
-    ~Scratch() {
-      for (void *q : p)
-        if (q) cudaFree(q);
-    }
-  } sc;
-  KMC_TRY(dalloc(reinterpret_cast<double **>(&sc.p[0]), sizeof(double) * 3 * n));
-  KMC_TRY(dalloc(reinterpret_cast<double **>(&sc.p[1]), sizeof(double) * 3 * B));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&sc.p[2]), sizeof(int32_t) * B));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&sc.p[3]), sizeof(int32_t) * B));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&sc.p[4]), sizeof(int32_t) * B * kmc::kRsaMaxConf));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&sc.p[5]), sizeof(int32_t)));
-  KMC_TRY(dalloc(reinterpret_cast<long long **>(&sc.p[6]), sizeof(long long)));
-  KMC_TRY(dalloc(reinterpret_cast<float4 **>(&sc.p[7]), sizeof(float4) * n));
-  KMC_CUDA(cudaMemsetAsync(sc.p[5], 0, sizeof(int32_t), c->stream));
   kmc::RsaArgs a;
   a.Rb = radius - 0.5 * diameter;
   a.d2 = diameter * diameter;
@@ -2536,14 +2537,38 @@ kmc_status kmc_regenerate_rsa(kmc_ctx *c, int32_t lys, double radius, double dia
   a.lys = lys;
   a.B = B;
   a.n = n;
-  a.pos = static_cast<double *>(sc.p[0]);
-  a.cand = static_cast<double *>(sc.p[1]);
-  a.clear = static_cast<int32_t *>(sc.p[2]);
-  a.nconf = static_cast<int32_t *>(sc.p[3]);
-  a.conf = static_cast<int32_t *>(sc.p[4]);
-  a.kept = static_cast<int32_t *>(sc.p[5]);
-  a.used = static_cast<long long *>(sc.p[6]);
-  a.posf = static_cast<float4 *>(sc.p[7]);
+  // cells of edge d, or wider where those would be more than 8 n + 64 (the factor
+  // keeps spheres closer than d in touching cells under the rounding of the cell
+  // index, 1e-13 relative at most)
+  {
+    const double side = std::cbrt(std::min(8.0 * n + 64.0, 1e9));
+    const double edge = std::max(diameter, 2.0 * a.Rb / side) * (1.0 + 1e-9);
+    a.inv_edge = 1.0 / edge;
+    a.dim = static_cast<int>(2.0 * a.Rb / edge) + 1;
+  }
+  Scratch sc;
+  const size_t cells = static_cast<size_t>(a.dim) * a.dim * a.dim;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) {
+      KMC_TRY(dalloc(&sc.p, sc.used));
+      sc.used = 0;
+    }
+    sc.take(&a.pos, 3ull * n);
+    sc.take(&a.cand, 3ull * B);
+    sc.take(&a.posf, n);
+    sc.take(&a.candf, B);
+    sc.take(&a.clear, B);
+    sc.take(&a.nconf, B);
+    sc.take(&a.conf, static_cast<size_t>(B) * kmc::kRsaMaxConf);
+    sc.take(&a.next_b, B);
+    sc.take(&a.next_k, n);
+    sc.take(&a.head_b, cells);
+    sc.take(&a.head_k, cells);
+    sc.take(&a.used, 1);
+    sc.take(&a.kept, 1);
+  }
+  KMC_CUDA(cudaMemsetAsync(a.kept, 0, sizeof(int32_t), c->stream));
+  KMC_CUDA(cudaMemsetAsync(a.head_k, 0xff, sizeof(int32_t) * cells, c->stream));
   // FP32 pre-screen: with centres within Rb of the origin, converting them
   // to FP32 (error <= u Rb per coordinate, u = 2^-24) and forming the squared
   // distance D^2 in FP32 errs by at most 4 sqrt(3) u Rb D + 5 u D^2; the

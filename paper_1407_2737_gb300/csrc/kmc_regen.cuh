@@ -148,103 +148,167 @@ __device__ __forceinline__ double rsa_d2(const double *p, const double *q) {
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// Spheres p (pf in FP32) and q closer than d. The FP32 squared distance settles
+// the pair unless it falls within the margin [d2_lo, d2_hi] around d^2, which
+// bounds its error for centres inside the ball; there the FP64 test of the
+// definition decides.
+__device__ __forceinline__ bool rsa_close(const RsaArgs &a, const double *p, const float4 &pf,
+                                          const double *q, const float4 &qf) {
+  const float dx = pf.x - qf.x, dy = pf.y - qf.y, dz = pf.z - qf.z;
+  const float d2f = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+  return d2f < a.d2_lo || (d2f <= a.d2_hi && rsa_d2(p, q) < a.d2);
+}
+
+// Cubic cells of edge at least d over the ball's box: spheres closer than d lie
+// in the same or in touching cells. Each cell heads a linked list of the kept
+// spheres in it and one of the batch's candidates; the order inside a list
+// varies, what is found in it does not.
+__device__ __forceinline__ int3 rsa_cell(const RsaArgs &a, const double *p) {
+  auto at = [&](double x) {
+    return min(max(static_cast<int>((x + a.Rb) * a.inv_edge), 0), a.dim - 1);
+  };
+  return make_int3(at(p[0]), at(p[1]), at(p[2]));
+}
+
+// f(j) for every entry j of the lists about cell c, until f returns true.
+template <typename F>
+__device__ __forceinline__ bool rsa_around(const RsaArgs &a, const int3 &c, const int32_t *head,
+                                           const int32_t *next, F f) {
+  for (int z = max(c.z - 1, 0); z <= min(c.z + 1, a.dim - 1); ++z)
+    for (int y = max(c.y - 1, 0); y <= min(c.y + 1, a.dim - 1); ++y)
+      for (int x = max(c.x - 1, 0); x <= min(c.x + 1, a.dim - 1); ++x)
+        for (int j = head[(z * a.dim + y) * a.dim + x]; j >= 0; j = next[j])
+          if (f(j)) return true;
+  return false;
+}
+
+__device__ __forceinline__ int rsa_index(const RsaArgs &a, const int3 &c) {
+  return (c.z * a.dim + c.y) * a.dim + c.x;
+}
+
+// Candidate k of the batch: drawn, and checked against the spheres that earlier
+// batches kept; if it clears them it joins its cell's list of candidates.
 __global__ void rsa_candidates_kernel(const RsaArgs a) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < a.B) rsa_candidate(a.Rb, a.seed, a.loop, a.c0 + k, a.lys, a.cand + 3 * k);
+  if (k >= a.B) return;
+  double p[3];
+  rsa_candidate(a.Rb, a.seed, a.loop, a.c0 + k, a.lys, p);
+  const float4 pf = make_float4(static_cast<float>(p[0]), static_cast<float>(p[1]),
+                                static_cast<float>(p[2]), 0.0f);
+  for (int q = 0; q < 3; ++q) a.cand[3 * k + q] = p[q];
+  a.candf[k] = pf;
+  const int3 c = rsa_cell(a, p);
+  const bool clash = rsa_around(a, c, a.head_k, a.next_k, [&](int j) {
+    return rsa_close(a, p, pf, a.pos + 3 * j, a.posf[j]);
+  });
+  a.clear[k] = clash ? 0 : 1;
+  if (!clash) a.next_b[k] = atomicExch(a.head_b + rsa_index(a, c), k);
 }
 
-// Block k: does candidate k clear every sphere kept by earlier batches, and
-// which earlier candidates of this batch lie closer than d. Against the kept
-// spheres an FP32 squared distance settles the pair unless it falls within
-// the margin [d2_lo, d2_hi] around d^2, which bounds the FP32 error for
-// centres inside the ball; there the FP64 test of the definition decides.
-__global__ void rsa_check_kernel(const RsaArgs a) {
-  __shared__ int s_nconf;
-  const int k = blockIdx.x;
-  const int kept = *a.kept;
+// The earlier candidates of the batch that candidate k clashes with (counted;
+// the first kRsaMaxConf listed).
+__global__ void rsa_conflicts_kernel(const RsaArgs a) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= a.B || !a.clear[k]) return;
   const double *p = a.cand + 3 * k;
-  const float px = static_cast<float>(p[0]), py = static_cast<float>(p[1]),
-              pz = static_cast<float>(p[2]);
-  bool clash = false;
-  for (int j = threadIdx.x; j < kept && !clash; j += blockDim.x) {
-    const float4 q = a.posf[j];
-    const float dx = px - q.x, dy = py - q.y, dz = pz - q.z;
-    const float d2f = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-    if (d2f < a.d2_lo)
-      clash = true;
-    else if (d2f <= a.d2_hi)
-      clash = rsa_d2(p, a.pos + 3 * j) < a.d2;
-  }
-  if (threadIdx.x == 0) s_nconf = 0;
-  clash = __syncthreads_or(clash);
-  if (!clash) {
-    for (int j = threadIdx.x; j < k; j += blockDim.x)
-      if (rsa_d2(p, a.cand + 3 * j) < a.d2) {
-        const int q = atomicAdd(&s_nconf, 1);
-        if (q < kRsaMaxConf) a.conf[k * kRsaMaxConf + q] = j;
-      }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    a.clear[k] = clash ? 0 : 1;
-    a.nconf[k] = s_nconf;
-  }
+  const float4 pf = a.candf[k];
+  int n = 0;
+  rsa_around(a, rsa_cell(a, p), a.head_b, a.next_b, [&](int j) {
+    if (j < k && rsa_close(a, p, pf, a.cand + 3 * j, a.candf[j])) {
+      if (n < kRsaMaxConf) a.conf[k * kRsaMaxConf + n] = j;
+      ++n;
+    }
+    return false;
+  });
+  a.nconf[k] = n;
 }
 
-// The batch in candidate order: a candidate that cleared the earlier batches
-// is kept unless a candidate kept earlier in this batch lies closer than d.
-// That is the sequential rule, candidate by candidate. The walk is one thread
-// on shared-memory copies (dynamic shared memory: rsa_resolve_smem(B) bytes);
-// the kept centres are then copied out by the whole block.
-__host__ __device__ constexpr size_t rsa_resolve_smem(int B) {
-  return static_cast<size_t>(B) * (3 + kRsaMaxConf) * sizeof(int32_t);
+// The sequential rule over the batch, by one block: a candidate that cleared the
+// earlier batches is kept unless one kept earlier in this batch lies closer
+// than d. Its fate is known once those of its earlier conflicts are: in rounds,
+// each decides every candidate whose conflicts are decided (the first undecided
+// one always is), until none is left. The rounds follow chains of conflicts,
+// a dozen or so, where a walk in candidate order took as many steps as
+// candidates. The kept ones' places follow from a scan in candidate order.
+__global__ void __launch_bounds__(1024) rsa_resolve_kernel(const RsaArgs a) {
+  extern __shared__ unsigned char s_state[];  // per candidate: 0 undecided, 1 kept, 2 not
+  __shared__ int s_sum[32];
+  volatile unsigned char *state = s_state;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // bit i of todo: this thread's candidate threadIdx.x + 1024 i is undecided
+  static_assert(kRsaMaxBatch <= 32 * 1024, "a thread's candidates are bits of one word");
+  unsigned todo = 0;
+  for (int i = 0, k = threadIdx.x; k < a.B; ++i, k += 1024) {
+    const int st = !a.clear[k] ? 2 : (a.nconf[k] == 0 ? 1 : 0);
+    state[k] = static_cast<unsigned char>(st);
+    todo |= static_cast<unsigned>(st == 0) << i;
+  }
+  __syncthreads();
+  for (;;) {
+    for (unsigned left = todo; left;) {
+      const int i = __ffs(left) - 1;
+      left &= left - 1;
+      const int k = threadIdx.x + 1024 * i;
+      bool wait = false, out = false;
+      auto meet = [&](int j) {
+        const unsigned char s = state[j];
+        out = out || s == 1;
+        wait = wait || s == 0;
+      };
+      const int nc = a.nconf[k];
+      if (nc <= kRsaMaxConf) {
+        for (int q = 0; q < nc && !out; ++q) meet(a.conf[k * kRsaMaxConf + q]);
+      } else {
+        const double *p = a.cand + 3 * k;
+        const float4 pf = a.candf[k];
+        rsa_around(a, rsa_cell(a, p), a.head_b, a.next_b, [&](int j) {
+          if (j < k && rsa_close(a, p, pf, a.cand + 3 * j, a.candf[j])) meet(j);
+          return out;
+        });
+      }
+      if (out || !wait) {
+        state[k] = out ? 2 : 1;
+        todo &= ~(1u << i);
+      }
+    }
+    if (!__syncthreads_or(todo != 0)) break;
+  }
+  // places in candidate order: thread t counts a run of consecutive candidates
+  const int per = (a.B + 1023) / 1024, k0 = threadIdx.x * per, k1 = min(a.B, k0 + per);
+  int own = 0;
+  for (int k = k0; k < k1; ++k) own += state[k] == 1;
+  int inc = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  if (lane == 31) s_sum[warp] = inc;
+  const int kept = *a.kept;
+  __syncthreads();
+  int before = 0, all = 0;
+  for (int w = 0; w < 32; ++w) {
+    before += w < warp ? s_sum[w] : 0;
+    all += s_sum[w];
+  }
+  int slot = kept + before + inc - own;
+  for (int k = k0; k < k1; ++k) {
+    const bool in = state[k] == 1 && slot < a.n;
+    a.clear[k] = in ? 1 + slot : 0;  // for rsa_place_kernel
+    if (in && ++slot == a.n) *a.used = a.c0 + k + 1;
+  }
+  if (threadIdx.x == 0) *a.kept = min(a.n, kept + all);
 }
 
-__global__ void rsa_resolve_kernel(const RsaArgs a) {
-  extern __shared__ int32_t rsa_sm[];
-  int32_t *s_clear = rsa_sm, *s_nconf = rsa_sm + a.B, *s_slot = rsa_sm + 2 * a.B;
-  int32_t *s_conf = rsa_sm + 3 * a.B;
-  __shared__ int32_t s_kept;
-  for (int k = threadIdx.x; k < a.B; k += blockDim.x) {
-    s_clear[k] = a.clear[k];
-    s_nconf[k] = a.nconf[k];
-    s_slot[k] = -1;
-  }
-  for (int q = threadIdx.x; q < a.B * kRsaMaxConf; q += blockDim.x) s_conf[q] = a.conf[q];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int kept = *a.kept;
-    for (int k = 0; k < a.B && kept < a.n; ++k) {
-      bool ok = s_clear[k] != 0;
-      if (ok) {
-        const int nc = s_nconf[k];
-        if (nc <= kRsaMaxConf) {
-          for (int q = 0; q < nc && ok; ++q) ok = s_slot[s_conf[k * kRsaMaxConf + q]] < 0;
-        } else {
-          for (int j = 0; j < k && ok; ++j)
-            ok = !(s_slot[j] >= 0 && rsa_d2(a.cand + 3 * k, a.cand + 3 * j) < a.d2);
-        }
-      }
-      if (ok) {
-        s_slot[k] = kept;
-        if (++kept == a.n) *a.used = a.c0 + k + 1;
-      }
-    }
-    s_kept = kept;
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < a.B; k += blockDim.x) {
-    const int sl = s_slot[k];
-    if (sl >= 0) {
-      const double x = a.cand[3 * k], y = a.cand[3 * k + 1], z = a.cand[3 * k + 2];
-      a.pos[3 * sl] = x;
-      a.pos[3 * sl + 1] = y;
-      a.pos[3 * sl + 2] = z;
-      a.posf[sl] = make_float4(static_cast<float>(x), static_cast<float>(y),
-                               static_cast<float>(z), 0.0f);
-    }
-  }
-  if (threadIdx.x == 0) *a.kept = s_kept;
+// The kept candidates into their places and into the lists of kept spheres.
+__global__ void rsa_place_kernel(const RsaArgs a) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= a.B || a.clear[k] == 0) return;
+  const int slot = a.clear[k] - 1;
+  const double *p = a.cand + 3 * k;
+  for (int q = 0; q < 3; ++q) a.pos[3 * slot + q] = p[q];
+  a.posf[slot] = a.candf[k];
+  a.next_k[slot] = atomicExch(a.head_k + rsa_index(a, rsa_cell(a, p)), slot);
 }
 
 }  // namespace kmc

@@ -2495,9 +2495,13 @@ cudaError_t launch_regen(const RegenArgs &a, cudaStream_t st) {
 
 cudaError_t launch_rsa_batch(const RsaArgs &a, cudaStream_t st) {
   if (a.B <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(
+      a.head_b, 0xff, sizeof(int32_t) * static_cast<size_t>(a.dim) * a.dim * a.dim, st);
+  if (e != cudaSuccess) return e;
   rsa_candidates_kernel<<<(a.B + 127) / 128, 128, 0, st>>>(a);
-  rsa_check_kernel<<<a.B, 128, 0, st>>>(a);
-  rsa_resolve_kernel<<<1, 1024, rsa_resolve_smem(a.B), st>>>(a);
+  rsa_conflicts_kernel<<<(a.B + 127) / 128, 128, 0, st>>>(a);
+  rsa_resolve_kernel<<<1, 1024, a.B, st>>>(a);
+  rsa_place_kernel<<<(a.B + 127) / 128, 128, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -2572,9 +2576,6 @@ cudaError_t init_device() {
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<4>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<8>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<16>);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(rsa_resolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(rsa_resolve_smem(kRsaMaxBatch)));
   return e;
 }
 

@@ -286,12 +286,18 @@ struct RsaArgs {
   float4 *posf;                // [n] the same in FP32 (x, y, z, 0), for the pre-screen
   float d2_lo, d2_hi;          // FP32 squared distances below d2_lo clash and above d2_hi
                                // clear for certain; in between the FP64 test decides
+  double inv_edge;             // cells: inverse edge, and how many along each side of
+  int32_t dim;                 // the box [-Rb, Rb]^3
+  int32_t *head_k, *next_k;    // [dim^3], [n] lists of the kept spheres (-1: end)
+  int32_t *head_b, *next_b;    // [dim^3], [B] lists of the batch's candidates
   double *cand;                // [B][3] scratch
-  int32_t *clear;              // [B] 1 if the candidate clears the earlier batches' spheres
+  float4 *candf;               // [B] the same in FP32
+  int32_t *clear;              // [B] 1 if the candidate clears the earlier batches' spheres;
+                               // once resolved, 1 + its place if it is kept, else 0
   int32_t *nconf;              // [B] earlier candidates of the batch closer than d
   int32_t *conf;               // [B][kRsaMaxConf] their indices
 };
-constexpr int kRsaMaxBatch = 2048;  // candidates per batch at most
+constexpr int kRsaMaxBatch = 32768;  // candidates per batch at most
 struct RegenArgs {
   int32_t off, n, lys, what;
   uint32_t loop;
