@@ -41,16 +41,16 @@ using kmc::SrcPair;
 
 constexpr int kMaxN = KMC_NOALLOC_MAX_N;
 constexpr int kMaxRec = kMaxN / 2;
-constexpr int kGroups = kMaxN / 32;
-constexpr int kChunkRec = 512;                                  // source records per item
-constexpr int kMaxSplit = (kMaxRec + kChunkRec - 1) / kChunkRec;
-constexpr int kMaxItems = kGroups * kMaxSplit;
+constexpr int kGroup = 64;                                      // targets per block, two per lane
+constexpr int kGroups = kMaxN / kGroup;
+constexpr int kMaxSplit = 16;                                   // source ranges per group
+constexpr int kMaxItems = 1024;                                 // blocks
 constexpr int kTile = 128;                                      // records per staged tile
 constexpr int kWarps = 4;
 constexpr size_t kRecBytes = sizeof(SrcPair) * kMaxRec;
 constexpr size_t kTgtBytes = sizeof(float4) * kMaxN;
-constexpr size_t kPartBytes = sizeof(float) * 6 * 32 * kMaxItems;  // (sum, error) x 3
-constexpr size_t kCntBytes = sizeof(int) * kGroups;
+constexpr size_t kPartBytes = sizeof(float) * 6 * kGroup * kMaxItems;  // (sum, error) x 3
+constexpr size_t kCntBytes = sizeof(int) * (kGroups + 4);       // per group; groups finished
 constexpr size_t kErrBytes = 16;                                // the error word, padded
 constexpr size_t kNoallocBytes = kRecBytes + kTgtBytes + kPartBytes + kCntBytes + kErrBytes;
 
@@ -97,7 +97,7 @@ __global__ void noalloc_pack(unsigned char *scratch, int n, const double *__rest
                              const double *__restrict__ m, const double *__restrict__ vol,
                              double cx, double cy, double cz, double inv_len, double w_scale) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kGroups) sc_cnt(scratch)[i] = 0;
+  if (i <= kGroups) sc_cnt(scratch)[i] = 0;
   if (i == 0) *sc_err(scratch) = 0;
   if (i >= n + (n & 1)) return;
   SrcPair &r = sc_rec(scratch)[i >> 1];
@@ -120,46 +120,85 @@ __global__ void noalloc_pack(unsigned char *scratch, int n, const double *__rest
   sc_tgt(scratch)[i] = make_float4(x, y, z, w);
 }
 
-// The records of one staged tile taken by this warp (every kWarps-th).
+// The records of one staged tile taken by this warp (every kWarps-th) against
+// the lane's two targets.
 template <bool MASK>
-__device__ __forceinline__ AccF32 tile_pairs(const ulonglong2 *__restrict__ sp, int cnt, int first,
-                                             f2 X, f2 Y, f2 Z) {
-  AccF32 acc;
-  acc.x = acc.y = acc.z = 0ull;
-#pragma unroll 2
+__device__ __forceinline__ void tile_pairs(const ulonglong2 *__restrict__ sp, int cnt, int first,
+                                           const f2 (&X)[2], const f2 (&Y)[2], const f2 (&Z)[2],
+                                           AccF32 (&acc)[2]) {
+#pragma unroll 8
   for (int r = first; r < cnt; r += kWarps) {
     ulonglong2 a, b, c, d;
     f2 e;
     kmc::load_record(sp, r, a, b, c, d, e);
-    kmc::pair_record<MASK>(a, b, c, d, e, X, Y, Z, acc);
+    kmc::pair_record<MASK>(a, b, c, d, e, X[0], Y[0], Z[0], acc[0]);
+    kmc::pair_record<MASK>(a, b, c, d, e, X[1], Y[1], Z[1], acc[1]);
   }
-  return acc;
 }
 
-// One block = 32 targets x one source range; the last block of a target group
-// adds the partial sums in split order and writes mu0 H_dip = bunit * b_dip.
-// A staging wait that runs out (after wait_ns) sets the error word; the
-// block's sums become NaN, so that the group's targets get NaN in B, and the
-// block still arrives, so that the group completes. stall_tx > 0 (a test of
+// Source ranges per group for G groups and nrec source records. Rough cycles:
+// an SM works a block's range off at 22.5 per record (64 targets, 18 packed
+// instructions per record and target at 0.8 of the pipe) plus 600; a block alone on
+// its SM takes 27 per record (one warp per scheduler) plus 2000 for its first
+// tile and epilogue; handing partial sums over costs 1500, and 30 for each. The
+// minimum over the ranges that the scratch holds fills the SMs where there are
+// few groups and evens out the last wave where there are many.
+int splits_for(int G, int nrec) {
+  constexpr int kSms = 152;
+  int best = 1;
+  double t_best = 0.0;
+  for (int s = 1; s <= kMaxSplit && G * s <= kMaxItems; ++s) {
+    const double r = static_cast<double>(nrec) / s;
+    if (s > 1 && r < 16.0) break;
+    const double per_sm = (G * s + kSms - 1) / kSms;
+    double t = per_sm * (22.5 * r + 600.0);
+    if (27.0 * r + 2000.0 > t) t = 27.0 * r + 2000.0;
+    if (s > 1) t += 1500.0 + 30.0 * s;
+    if (s == 1 || t < t_best) {
+      best = s;
+      t_best = t;
+    }
+  }
+  return best;
+}
+
+// One block = 64 targets (two per lane: each staged record feeds two chains) x
+// one source range; the last block of a target group adds the partial sums in
+// split order and writes mu0 H_dip = bunit * b_dip, and the last group to finish
+// writes the status. A staging wait that runs out (after wait_ns) sets the error
+// word; the block's sums become NaN, so that the group's targets get NaN in B, and
+// the block still arrives, so that the group completes. stall_tx > 0 (a test of
 // that path) makes every tile expect that many bytes more than its copy
-// delivers, so that every wait runs out while no copy is left unfinished.
-__global__ void __launch_bounds__(kWarps * 32)
+// delivers, so that every wait runs out while no copy is left unfinished. Bound:
+// the FP32 pipe, as kmc_step_f32_tn, whose pair loop this is.
+// 8192 NPs: 52 us (7 ranges, 896 blocks) against 58 for one target per lane in ranges
+// of 512 records, the call 57 against 65; 3000 NPs 18.6 against 23.6 us.
+__global__ void __launch_bounds__(kWarps * 32, 4)
     noalloc_field(unsigned char *scratch, int n, int nsplit, double bunit,
-                  double *__restrict__ B, uint32_t stall_tx, unsigned long long wait_ns) {
+                  double *__restrict__ B, int32_t *__restrict__ status, uint32_t stall_tx,
+                  unsigned long long wait_ns) {
   __shared__ __align__(128) ulonglong2 buf[2][kTile * kmc::kRecU2];
-  __shared__ float wp[kWarps][6][32];
+  __shared__ float wp[kWarps][12][32];
   __shared__ uint64_t bar[2];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
-  const int t0 = 32 * g, nt = min(32, n - t0);
+  const int t0 = kGroup * g, nt = min(kGroup, n - t0);
   const int nrec = (n + 1) / 2;
   const int j0 = static_cast<int>(static_cast<long long>(split) * nrec / nsplit);
   const int j1 = static_cast<int>(static_cast<long long>(split + 1) * nrec / nsplit);
   const int own0 = t0 >> 1, own1 = (t0 + nt - 1) >> 1;
-  const float4 p = sc_tgt(scratch)[t0 + min(lane, nt - 1)];
-  const f2 X = kmc::pk(p.x, p.x), Y = kmc::pk(p.y, p.y), Z = kmc::pk(p.z, p.z);
-  float s3[3] = {0.f, 0.f, 0.f}, c3[3] = {0.f, 0.f, 0.f};
+  f2 X[2], Y[2], Z[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {  // lanes past the last target repeat it
+    const float4 p = sc_tgt(scratch)[t0 + min(32 * k + lane, nt - 1)];
+    X[k] = kmc::pk(p.x, p.x);
+    Y[k] = kmc::pk(p.y, p.y);
+    Z[k] = kmc::pk(p.z, p.z);
+  }
+  float s6[6], c6[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) s6[c] = c6[c] = 0.f;
   const SrcPair *src = sc_rec(scratch);
   int32_t *err = sc_err(scratch);
   const int ntiles = (j1 - j0 + kTile - 1) / kTile;
@@ -184,12 +223,19 @@ __global__ void __launch_bounds__(kWarps * 32)
     const bool ok = kmc::mbar_wait_bounded(&bar[t & 1], (t >> 1) & 1, err, wait_ns);
     if (ok) {
       const int r0 = j0 + t * kTile, cnt = min(kTile, j1 - r0);
-      const AccF32 acc = (r0 <= own1 && own0 < r0 + cnt)
-                             ? tile_pairs<true>(buf[t & 1], cnt, warp, X, Y, Z)
-                             : tile_pairs<false>(buf[t & 1], cnt, warp, X, Y, Z);
-      kmc::kahan_add(s3[0], c3[0], kmc::hsum(acc.x));
-      kmc::kahan_add(s3[1], c3[1], kmc::hsum(acc.y));
-      kmc::kahan_add(s3[2], c3[2], kmc::hsum(acc.z));
+      AccF32 acc[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) acc[k].x = acc[k].y = acc[k].z = 0ull;
+      if (r0 <= own1 && own0 < r0 + cnt)
+        tile_pairs<true>(buf[t & 1], cnt, warp, X, Y, Z, acc);
+      else
+        tile_pairs<false>(buf[t & 1], cnt, warp, X, Y, Z, acc);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        kmc::kahan_add(s6[3 * k + 0], c6[3 * k + 0], kmc::hsum(acc[k].x));
+        kmc::kahan_add(s6[3 * k + 1], c6[3 * k + 1], kmc::hsum(acc[k].y));
+        kmc::kahan_add(s6[3 * k + 2], c6[3 * k + 2], kmc::hsum(acc[k].z));
+      }
     }
     if (!__syncthreads_and(ok)) {
       if (threadIdx.x == 0) kmc::drain_copies(bar, t, ntiles, wait_ns);
@@ -203,68 +249,71 @@ __global__ void __launch_bounds__(kWarps * 32)
   }
   if (failed) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) s3[c] = __int_as_float(0x7fc00000);  // NaN
+    for (int c = 0; c < 6; ++c) s6[c] = __int_as_float(0x7fc00000);  // NaN
   }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    wp[warp][c][lane] = s3[c];
-    wp[warp][3 + c][lane] = -c3[c];
+  for (int c = 0; c < 6; ++c) {
+    wp[warp][c][lane] = s6[c];
+    wp[warp][6 + c][lane] = -c6[c];
   }
   __syncthreads();
+  // warp k < 2: the lane's target 32 k + lane
   float hi[3], lo[3];
-  if (warp == 0) {
+  if (warp < 2) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       float s = 0.f, e = 0.f;
       for (int w = 0; w < kWarps; ++w) {
-        kmc::neumaier_add(s, e, wp[w][c][lane]);
-        e += wp[w][3 + c][lane];
+        kmc::neumaier_add(s, e, wp[w][3 * warp + c][lane]);
+        e += wp[w][6 + 3 * warp + c][lane];
       }
       hi[c] = s;
       lo[c] = e;
     }
-    if (nsplit > 1) {
-      float *part = sc_part(scratch) + static_cast<size_t>(blockIdx.x) * 6 * 32;
+  }
+  if (nsplit > 1) {
+    constexpr size_t kItem = 6 * kGroup;  // floats: [2 parts][6][32]
+    if (warp < 2) {
+      float *part = sc_part(scratch) + blockIdx.x * kItem + warp * 192;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         __stcg(part + c * 32 + lane, hi[c]);
         __stcg(part + (3 + c) * 32 + lane, lo[c]);
       }
-      __threadfence();
     }
-  }
-  if (nsplit > 1) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&sc_cnt(scratch)[g], 1) == nsplit - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (warp == 0) {
-      const float *base = sc_part(scratch) + static_cast<size_t>(blockIdx.x - split) * 6 * 32;
+    if (!kmc::arrive_last(&sc_cnt(scratch)[g], nsplit, &s_last)) return;
+    if (warp < 2) {
+      const float *base = sc_part(scratch) + (blockIdx.x - split) * kItem + warp * 192;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         float s = 0.f, e = 0.f;
+#pragma unroll 4
         for (int q = 0; q < nsplit; ++q) {
-          kmc::neumaier_add(s, e, __ldcg(base + (q * 6 + c) * 32 + lane));
-          e += __ldcg(base + (q * 6 + 3 + c) * 32 + lane);
+          kmc::neumaier_add(s, e, __ldcg(base + q * kItem + c * 32 + lane));
+          e += __ldcg(base + q * kItem + (3 + c) * 32 + lane);
         }
         hi[c] = s;
         lo[c] = e;
       }
-      if (lane == 0) sc_cnt(scratch)[g] = 0;
     }
   }
-  if (warp == 0 && lane < nt) {
+  const int t = 32 * warp + lane;
+  if (warp < 2 && t < nt) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) B[3 * (t0 + lane) + c] = bunit * static_cast<double>(hi[c] + lo[c]);
+    for (int c = 0; c < 3; ++c) B[3 * (t0 + t) + c] = bunit * static_cast<double>(hi[c] + lo[c]);
   }
-}
-
-// The call's status for the caller: KMC_OK, or KMC_ETIMEOUT if a wait ran out.
-__global__ void noalloc_status(const unsigned char *scratch, int32_t *status) {
-  const int32_t e = *reinterpret_cast<const int32_t *>(scratch + kRecBytes + kTgtBytes +
-                                                       kPartBytes + kCntBytes);
-  *status = (e & kmc::kErrTimeout) ? KMC_ETIMEOUT : KMC_OK;
+  // the call's status once every group is done: KMC_OK, or KMC_ETIMEOUT if a wait ran out
+  if (status && threadIdx.x == 0) {
+    const int groups = (n + kGroup - 1) / kGroup;
+    int32_t done;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+                 : "=r"(done)
+                 : "l"(sc_cnt(scratch) + kGroups)
+                 : "memory");
+    if (done == groups - 1)
+      *status = (*reinterpret_cast<volatile int32_t *>(err) & kmc::kErrTimeout) ? KMC_ETIMEOUT
+                                                                               : KMC_OK;
+  }
 }
 
 kmc_status fail(kmc_status s, const char *msg, cudaError_t e = cudaSuccess) {
@@ -390,25 +439,20 @@ kmc_status kmc_dipolar_field_noalloc(int32_t n, const double *pos, const double 
   unsigned char *scratch = static_cast<unsigned char *>(addr);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int nrec = (n + 1) / 2;
-  const int nsplit = (nrec + kChunkRec - 1) / kChunkRec;
-  const int groups = (n + 31) / 32;
+  const int groups = (n + kGroup - 1) / kGroup;
+  const int nsplit = splits_for(groups, nrec);
   const double inv_len = 1.0 / length;
   const double w_scale = 1.0 / (4.0 * kPi * length * length * length);
   const int packed = n + (n & 1);
-  const int threads = packed > kGroups ? packed : kGroups;
+  const int threads = packed > kGroups ? packed : kGroups + 1;
   noalloc_pack<<<(threads + 255) / 256, 256, 0, st>>>(scratch, n, pos, m, vol, center[0],
                                                       center[1], center[2], inv_len, w_scale);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(KMC_ECUDA, "packing kernel launch failed", e);
-  noalloc_field<<<groups * nsplit, kWarps * 32, 0, st>>>(scratch, n, nsplit, kMu0 * Ms, B,
+  noalloc_field<<<groups * nsplit, kWarps * 32, 0, st>>>(scratch, n, nsplit, kMu0 * Ms, B, status,
                                                          stall_tx, wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(KMC_ECUDA, "field kernel launch failed", e);
-  if (status) {
-    noalloc_status<<<1, 1, 0, st>>>(scratch, status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(KMC_ECUDA, "status kernel launch failed", e);
-  }
   return KMC_OK;
 }
 
