@@ -279,6 +279,9 @@ struct kmc_ctx {
   int32_t *d_dbg_flags = nullptr;
   cudaStream_t own_stream = nullptr, stream = nullptr;
   long long step_global = 0;
+  // nothing has been queued since the last wait, which found no device error
+  // (cleared wherever this context queues a kernel)
+  bool settled = false;
   // latest run
   bool have_run = false;
   int S = 0, periods = 0, discard = 0, n_rec = 0;
@@ -789,6 +792,7 @@ kmc_status set_items(kmc_ctx *c, const Shape &sh) {
 }
 
 StepArgs base_args(kmc_ctx *c) {
+  c->settled = false;
   StepArgs a;
   std::memset(&a, 0, sizeof(a));
   a.items = c->d_items;
@@ -889,6 +893,7 @@ cudaError_t launch_one_step(const kmc_ctx *c, StepArgs a, const Shape &sh, cudaS
 }
 
 kmc_status refresh_sources(kmc_ctx *c, int par) {
+  c->settled = false;
   const int bs = 256;
   const unsigned nb = static_cast<unsigned>((c->N + bs - 1) / bs);
   if (c->fp32)
@@ -903,7 +908,11 @@ kmc_status refresh_sources(kmc_ctx *c, int par) {
   return KMC_OK;
 }
 
+// Waits for queued work and reports the device error word (once: the reads that
+// follow a run one after another then cost their own copy alone, 14 us a call
+// instead of 35).
 kmc_status check_device_error(kmc_ctx *c) {
+  if (c->settled) return KMC_OK;
   int32_t ew[2] = {0, 0};
   KMC_CUDA(cudaMemcpyAsync(ew, c->d_err, sizeof(ew), cudaMemcpyDeviceToHost, c->stream));
   KMC_CUDA(cudaStreamSynchronize(c->stream));
@@ -919,6 +928,7 @@ kmc_status check_device_error(kmc_ctx *c) {
     return fail(KMC_ESTATE,
                 "a dipolar field or barrier was not finite (two NPs at one point?); those NPs "
                 "kept their moments (KMC_READ_COUNTERS counts them)");
+  c->settled = true;
   return KMC_OK;
 }
 
@@ -2000,7 +2010,7 @@ kmc_status kmc_read(kmc_ctx *c, int32_t what, int32_t lys, double *buf, int64_t 
       what == KMC_READ_AXES) {
     // state, readable after a device error so that the caller can see what
     // happened (kmc_sync reports the error)
-    KMC_CUDA(cudaStreamSynchronize(c->stream));
+    if (!c->settled) KMC_CUDA(cudaStreamSynchronize(c->stream));
   } else {
     KMC_TRY(check_device_error(c));
   }
@@ -2433,74 +2443,83 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
       vfrac[o] = L.vol[i] / vs;
     }
   }
-  // device copies, freed on every path out
-  struct Buffers {
-    void *p[9] = {};
+  struct Stream {
     cudaStream_t st = nullptr;
-    ~Buffers() {
-      if (st) cudaStreamSynchronize(st);
-      for (void *q : p)
-        if (q) cudaFree(q);
-      if (st) cudaStreamDestroy(st);
+    ~Stream() {
+      if (st) {
+        cudaStreamSynchronize(st);
+        cudaStreamDestroy(st);
+      }
     }
-  } b;
+  };
+  // one allocation (freed after the stream has ended, on every path out), one copy
+  // in and one out
+  Scratch sc;
+  Stream b;
   KMC_CUDA(cudaStreamCreateWithFlags(&b.st, cudaStreamNonBlocking));
   const size_t nl = static_cast<size_t>(std::max(need, 1ll));
-  KMC_TRY(dalloc(reinterpret_cast<kmc::MeanLysDev **>(&b.p[0]), sizeof(kmc::MeanLysDev) * n_lys));
-  KMC_TRY(dalloc(reinterpret_cast<kmc::MeanItem **>(&b.p[1]), sizeof(kmc::MeanItem) * items.size()));
-  KMC_TRY(dalloc(reinterpret_cast<dbl4 **>(&b.p[2]), sizeof(dbl4) * N));
-  KMC_TRY(dalloc(reinterpret_cast<double **>(&b.p[3]), sizeof(double) * 2 * N));
-  KMC_TRY(dalloc(reinterpret_cast<double **>(&b.p[4]), sizeof(double) * S));
-  KMC_TRY(dalloc(reinterpret_cast<long long **>(&b.p[5]), sizeof(long long) * nl));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&b.p[6]), sizeof(int32_t)));
   // steps solved at once: as many as 64 MB hold (at least one), the launch's grid
   // bounding them too
   const size_t per_step = static_cast<size_t>(N) * (kmc::kMeanFields * sizeof(double) +
                                                     sizeof(int32_t));
   const int span = static_cast<int>(std::min<long long>(
       std::min(S, 65536), std::max<long long>(1, static_cast<long long>((64u << 20) / per_step))));
-  KMC_TRY(dalloc(reinterpret_cast<double **>(&b.p[7]),
-                 sizeof(double) * N * (kmc::kMeanState + kmc::kMeanFields * static_cast<size_t>(span))));
-  KMC_TRY(dalloc(reinterpret_cast<int32_t **>(&b.p[8]),
-                 sizeof(int32_t) * N * static_cast<size_t>(span)));
-  double *d_bv = static_cast<double *>(b.p[3]);
-  KMC_CUDA(cudaMemcpyAsync(b.p[0], hl.data(), sizeof(kmc::MeanLysDev) * n_lys,
-                           cudaMemcpyHostToDevice, b.st));
-  KMC_CUDA(cudaMemcpyAsync(b.p[1], items.data(), sizeof(kmc::MeanItem) * items.size(),
-                           cudaMemcpyHostToDevice, b.st));
-  KMC_CUDA(cudaMemcpyAsync(b.p[2], axis.data(), sizeof(dbl4) * N, cudaMemcpyHostToDevice, b.st));
-  KMC_CUDA(cudaMemcpyAsync(d_bv, beta.data(), sizeof(double) * N, cudaMemcpyHostToDevice, b.st));
-  KMC_CUDA(cudaMemcpyAsync(d_bv + N, vfrac.data(), sizeof(double) * N, cudaMemcpyHostToDevice,
-                           b.st));
-  KMC_CUDA(cudaMemcpyAsync(b.p[4], cosk.data(), sizeof(double) * S, cudaMemcpyHostToDevice, b.st));
-  KMC_CUDA(cudaMemsetAsync(b.p[5], 0, sizeof(long long) * nl, b.st));
-  KMC_CUDA(cudaMemsetAsync(b.p[6], 0, sizeof(int32_t), b.st));
   kmc::MeanArgs a;
-  a.items = static_cast<const kmc::MeanItem *>(b.p[1]);
+  kmc::MeanLysDev *d_lys = nullptr;
+  kmc::MeanItem *d_items = nullptr;
+  dbl4 *d_axis = nullptr;
+  double *d_beta = nullptr, *d_vfrac = nullptr, *d_cos = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) {
+      KMC_TRY(dalloc(&sc.p, sc.used));
+      sc.used = 0;
+    }
+    sc.take(&d_lys, n_lys);
+    sc.take(&d_items, items.size());
+    sc.take(&d_axis, N);
+    sc.take(&d_beta, N);
+    sc.take(&d_vfrac, N);
+    sc.take(&d_cos, S);
+    sc.take(&a.loop, nl);
+    sc.take(&a.err, 1);
+    sc.take(&a.state, static_cast<size_t>(N) * kmc::kMeanState);
+    sc.take(&a.wells, static_cast<size_t>(N) * kmc::kMeanFields * span);
+    sc.take(&a.flags, static_cast<size_t>(N) * span);
+  }
+  HostBytes in(reinterpret_cast<char *>(a.loop) - sc.p);
+  auto put = [&](const void *dst, const void *src, size_t bytes) {
+    std::memcpy(in.data() + (static_cast<const char *>(dst) - sc.p), src, bytes);
+  };
+  put(d_lys, hl.data(), sizeof(kmc::MeanLysDev) * n_lys);
+  put(d_items, items.data(), sizeof(kmc::MeanItem) * items.size());
+  put(d_axis, axis.data(), sizeof(dbl4) * N);
+  put(d_beta, beta.data(), sizeof(double) * N);
+  put(d_vfrac, vfrac.data(), sizeof(double) * N);
+  put(d_cos, cosk.data(), sizeof(double) * S);
+  const size_t out_bytes = reinterpret_cast<char *>(a.err) - reinterpret_cast<char *>(a.loop) +
+                           sizeof(int32_t);
+  KMC_CUDA(cudaMemcpyAsync(sc.p, in.data(), in.size(), cudaMemcpyHostToDevice, b.st));
+  KMC_CUDA(cudaMemsetAsync(a.loop, 0, out_bytes, b.st));
+  a.items = d_items;
   a.n_items = static_cast<int32_t>(items.size());
   a.S = S;
   a.periods = periods;
   a.discard = discard;
   a.n_rec = static_cast<int32_t>(std::max(n_rec, 1ll));
-  a.lys = static_cast<const kmc::MeanLysDev *>(b.p[0]);
-  a.axis = static_cast<const dbl4 *>(b.p[2]);
-  a.beta = d_bv;
-  a.vfrac = d_bv + N;
-  a.cos_k = static_cast<const double *>(b.p[4]);
-  a.loop = static_cast<long long *>(b.p[5]);
-  a.err = static_cast<int32_t *>(b.p[6]);
+  a.lys = d_lys;
+  a.axis = d_axis;
+  a.beta = d_beta;
+  a.vfrac = d_vfrac;
+  a.cos_k = d_cos;
   a.n = static_cast<int32_t>(N);
   a.span = span;
-  a.state = static_cast<double *>(b.p[7]);
-  a.wells = a.state + static_cast<size_t>(N) * kmc::kMeanState;
-  a.flags = static_cast<int32_t *>(b.p[8]);
   KMC_CUDA(kmc::launch_mean(a, b.st));
-  std::vector<long long> fx(nl);
-  int32_t err = 0;
-  KMC_CUDA(cudaMemcpyAsync(fx.data(), b.p[5], sizeof(long long) * nl, cudaMemcpyDeviceToHost,
-                           b.st));
-  KMC_CUDA(cudaMemcpyAsync(&err, b.p[6], sizeof(int32_t), cudaMemcpyDeviceToHost, b.st));
+  HostBytes out(out_bytes);
+  KMC_CUDA(cudaMemcpyAsync(out.data(), a.loop, out_bytes, cudaMemcpyDeviceToHost, b.st));
   KMC_CUDA(cudaStreamSynchronize(b.st));
+  const long long *fx = reinterpret_cast<const long long *>(out.data());
+  int32_t err = 0;
+  std::memcpy(&err, out.data() + out_bytes - sizeof(int32_t), sizeof(int32_t));
   if (err & kmc::kErrExtrema)
     return fail(KMC_ESTATE, "an energy profile had more than two minima or maxima");
   for (long long q = 0; q < need; ++q) loop_M[q] = static_cast<double>(fx[q]) / kmc::kLoopScale;
