@@ -180,7 +180,7 @@ __device__ __forceinline__ void segment_scan(EpiShared<R> &sm, const GridTables<
     pf.bc = bc;
     pf.bs = bs;
     const SignProfile sp(k2, bc, bs);
-    const int seg = (kGrid + nw - 1) / nw;
+    const int seg = ((kGrid + nw - 1) / nw + 1) & ~1;  // even: the packed pass
     const int j0 = warp * seg, len = min(kGrid, j0 + seg) - j0;
     if (len <= 0) return;
     const unsigned long long neg = fp64_signs(tab, pf, sp, j0, len);
@@ -239,7 +239,7 @@ __device__ __forceinline__ void segment_scan(EpiShared<R> &sm, const GridTables<
       for (int sg = warp; sg < nseg; sg += nw) scan(sg * seg, seg);
     }
   } else {
-    const int seg = (kGrid + nw - 1) / nw;
+    const int seg = ((kGrid + nw - 1) / nw + 1) & ~1;  // even: the packed pass
     const int j0 = warp * seg, len = min(kGrid, j0 + seg) - j0;
     if (len > 0) scan(j0, len);
   }
@@ -491,13 +491,23 @@ struct Decision {
 };
 
 // e^x for an exponent x held in FP64: x log2(e) = n + f exactly split into an
-// integer n and a fraction f in [0, 1); 2^f in FP32, then scaled by 2^n.
+// integer n and a fraction f in [0, 1); 2^f in FP32, then scaled by 2^n. The
+// split adds 1.5 2^52 rounding down, which leaves floor in the low word, where
+// floor(), its conversions and ldexpf made a longer chain (0.4 to 1 % of a step).
 __device__ __forceinline__ float exp_fp64_arg(double x) {
+  constexpr double kShift = 6755399441055744.0;  // 1.5 2^52
   const double y = x * 1.4426950408889634073599;  // log2(e)
-  if (y < -160.0) return 0.0f;
-  const double n = floor(y);
-  const float r = exp2f(static_cast<float>(y - n));
-  return ldexpf(r, static_cast<int>(fmin(n, 200.0)));
+  const float yf = static_cast<float>(y);
+  if (yf < -160.0f) return 0.0f;
+  if (yf > 200.0f) return INFINITY;  // beyond FP32 (2^128 and more)
+  const double t = __dadd_rd(y, kShift);
+  const int n = __double2loint(t);
+  const float r = exp2f(static_cast<float>(y - (t - kShift)));
+  // r 2^n, r in [1, 2]: two exact scalings and one that rounds, as ldexpf's
+  const int m = max(n, -126);
+  const float lo = __int_as_float((max(n - m, -126) + 127) << 23);  // 2^(n - m) <= 1
+  if (m > 127) return INFINITY;
+  return r * __int_as_float((m + 127) << 23) * lo;
 }
 
 // Steps v-vii for target t: basins, barrier (FP64 polish near the switching
@@ -522,13 +532,21 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
     cnt = cnt < 0 ? 0 : 4;
   }
   int nmin = 0, nmax = 0, imin0 = 0, imin1 = 0, imax0 = 0, imax1 = 0;
-  for (int q = 0; q < cnt; ++q) {
-    if (sm.dq[t][q] < R(0)) {
-      if (nmin == 0) imin0 = q; else imin1 = q;
-      ++nmin;
-    } else {
-      if (nmax == 0) imax0 = q; else imax1 = q;
-      ++nmax;
+  if ((cnt & 1) == 0 && !o.bad) {  // in grid order minima and maxima alternate
+    nmin = nmax = cnt >> 1;
+    if (cnt > 0) imin0 = sm.dq[t][0] < R(0) ? 0 : 1;
+    imax0 = 1 - imin0;
+    imin1 = imin0 + 2;
+    imax1 = imax0 + 2;
+  } else {
+    for (int q = 0; q < cnt; ++q) {
+      if (sm.dq[t][q] < R(0)) {
+        if (nmin == 0) imin0 = q; else imin1 = q;
+        ++nmin;
+      } else {
+        if (nmax == 0) imax0 = q; else imax1 = q;
+        ++nmax;
+      }
     }
   }
   if (nmin > 2 || nmax > 2) {
@@ -556,7 +574,9 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
   const R e3 = fmin(sm.en[t][imax0], sm.en[t][imax1]);
   double dEa = static_cast<double>(e3 - sm.en[t][wa]);
   double dEb = static_cast<double>(e3 - sm.en[t][wb]);
-  if (MIXED && fmin(dEa, dEb) < 1e-3 * static_cast<double>(sm.k[t])) {
+  // (for FP32 values, below 1e-3 k in FP64 is below it rounded up to FP32)
+  if (MIXED && fminf(static_cast<float>(e3 - sm.en[t][wa]), static_cast<float>(e3 - sm.en[t][wb])) <
+                   __double2float_ru(1e-3 * static_cast<double>(sm.k[t]))) {
     // Near the switching field E3 - E_a cancels: the energies of the two wells
     // and of the lower maximum are taken again in FP64 at the FP32 roots (the
     // energy is stationary there, so the root's FP32 error enters squared).
@@ -672,22 +692,6 @@ struct UpdateSync {
       asm volatile("bar.sync %0, %1;" ::"r"(1 + gid), "n"(GROUP * 32) : "memory");
     }
   }
-  static __device__ __forceinline__ bool sync_or(int gid, bool p) {
-    if constexpr (GROUP == 0) {
-      return __syncthreads_or(p) != 0;
-    } else {
-      uint32_t r;
-      asm volatile(
-          "{\n\t.reg .pred q, o;\n\t"
-          "setp.ne.u32 q, %1, 0;\n\t"
-          "bar.red.or.pred o, %2, %3, q;\n\t"
-          "selp.u32 %0, 1, 0, o;\n\t}"
-          : "=r"(r)
-          : "r"(static_cast<uint32_t>(p)), "r"(1 + gid), "n"(GROUP * 32)
-          : "memory");
-      return r != 0;
-    }
-  }
 };
 
 template <typename V, bool MIXED, bool WARP = false, int GROUP = 0>
@@ -740,9 +744,11 @@ __device__ __forceinline__ void block_update(
     segment_scan<R, (GROUP > 0 && GROUP < 4)>(sm, tab, warp, nw, lane, nt);
     Sync::sync(gid);
     if constexpr (MIXED) {
-      noisy = warp == 0 && lane < nt && (sm.cnt[lane] > 4 || a.force_rescan);
-      if (Sync::sync_or(gid, noisy)) {
-        if (noisy) rescan_fp64(sm, lane);
+      // every warp reads the same counts, so all of them take the same branch
+      noisy = lane < nt && (sm.cnt[lane] > 4 || a.force_rescan);
+      if (__any_sync(0xffffffffu, noisy)) {
+        Sync::sync(gid);  // the counts are read before they are replaced
+        if (warp == 0 && noisy) rescan_fp64(sm, lane);
         Sync::sync(gid);
       }
     }
