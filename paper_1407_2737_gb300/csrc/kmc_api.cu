@@ -154,13 +154,17 @@ struct Shape {
   // 1: the whole field period as one persistent cooperative launch (FP32, one
   // target per lane) with a grid barrier after each step
   int persist = 0;
+  // 1: the whole field period of lysosomes of up to 512 NPs as one launch, a
+  // thread-block cluster per lysosome (the autotuner's alone; FP32, warps = 8,
+  // chunk = 0)
+  int clu = 0;
   // symmetric form of FP64 contexts, the autotuner's alone: parts per cell pair
   // (1, 2, 4, 8 or 16; warps = 4, tile = 32, chunk = 0); 0 = the ordered kernel
   int f64 = 0;
   bool operator==(const Shape &o) const {
     return warps == o.warps && tile == o.tile && chunk == o.chunk && tpl == o.tpl &&
            rpl == o.rpl && sym == o.sym && cl == o.cl && supd == o.supd && persist == o.persist &&
-           f64 == o.f64 && bal == o.bal;
+           f64 == o.f64 && bal == o.bal && clu == o.clu;
   }
 };
 
@@ -268,6 +272,7 @@ struct kmc_ctx {
   // persistent period: the steps' cosines and the grid barrier's counters
   double *d_cosk = nullptr;
   size_t cosk_cap = 0;
+  int cosk_steps = 0;  // steps of the table's period (0: none yet)
   uint32_t *d_gbar = nullptr;
   int tpl_mode = 0;            // targets per lane: 0 = the autotuner's choice, else 1, 2 or 3
   int rpl_mode = 0;            // replicas per lane: 0 = the autotuner's choice, 1 = off, 2 or 4
@@ -715,6 +720,10 @@ kmc_status grow(kmc_ctx *c, T **p, size_t *cap, size_t need) {
 }
 
 kmc_status set_items(kmc_ctx *c, const Shape &sh) {
+  if (sh.clu) {  // its blocks need no items
+    c->items_shape = sh;
+    return KMC_OK;
+  }
   if (c->items_shape == sh && (sh.sym ? c->d_sitems != nullptr
                                       : sh.f64 ? c->d_fitems != nullptr : c->d_items != nullptr))
     return KMC_OK;
@@ -840,6 +849,7 @@ StepArgs base_args(kmc_ctx *c) {
 // The persistent period's cosine table for `steps` steps (the values the
 // per-step launches of a period graph receive) and its barrier counters.
 kmc_status prepare_persist(kmc_ctx *c, int steps) {
+  if (c->cosk_steps == steps) return KMC_OK;
   if (!c->d_gbar) KMC_TRY(dalloc(&c->d_gbar, 2 * sizeof(uint32_t)));
   if (static_cast<size_t>(steps) > c->cosk_cap) {
     if (c->d_cosk) cudaFree(c->d_cosk);
@@ -848,11 +858,13 @@ kmc_status prepare_persist(kmc_ctx *c, int steps) {
     KMC_TRY(dalloc(&c->d_cosk, sizeof(double) * steps));
     c->cosk_cap = static_cast<size_t>(steps);
   }
+  c->cosk_steps = 0;
   std::vector<double> cs(static_cast<size_t>(steps));
   for (int k = 0; k < steps; ++k) cs[k] = std::cos(2.0 * kPi * k / steps);
   KMC_CUDA(cudaMemcpyAsync(c->d_cosk, cs.data(), sizeof(double) * cs.size(),
                            cudaMemcpyHostToDevice, c->stream));
   KMC_CUDA(cudaStreamSynchronize(c->stream));
+  c->cosk_steps = steps;
   return KMC_OK;
 }
 
@@ -866,6 +878,21 @@ cudaError_t launch_period(kmc_ctx *c, StepArgs a, const Shape &sh, int steps) {
   return e;
 }
 
+int max_lysosome(const kmc_ctx *c) {
+  int n = 0;
+  for (int x : c->n) n = std::max(n, x);
+  return n;
+}
+
+// One cluster launch of `steps` steps, with the cosine table (prepare_persist)
+// or, without, a.cos_k.
+cudaError_t launch_cluster(const kmc_ctx *c, StepArgs a, int steps, bool table) {
+  const int n = max_lysosome(c);
+  a.S = steps;
+  a.cosk = table ? c->d_cosk : nullptr;
+  return kmc::launch_cluster(a, (n + kmc::kTargets - 1) / kmc::kTargets, n, c->stream);
+}
+
 // Chains of the current items (the symmetric forms have their own cuts).
 int n_chains_of(const kmc_ctx *c, const Shape &sh) {
   return static_cast<int>(sh.sym ? c->sym_cut_items.size()
@@ -875,6 +902,7 @@ int n_chains_of(const kmc_ctx *c, const Shape &sh) {
 // One step of every item of a (all chains, one stream), shape sh.
 cudaError_t launch_one_step(const kmc_ctx *c, StepArgs a, const Shape &sh, cudaStream_t st,
                             bool pdl) {
+  if (sh.clu) return launch_cluster(c, a, 1, false);
   if (sh.sym) {
     a.sitems = c->d_sitems;
     a.supd = c->d_supd;
@@ -951,6 +979,10 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
   if (s.persist != 0 && (s.persist != 1 || !c->fp32 || s.tpl != 1 || s.rpl != 1 || s.sym != 0 ||
                          s.cl != 0 || (s.warps != 4 && s.warps != 8)))
     return false;
+  if (s.clu != 0)
+    return c->fp32 && s.clu == 1 && s.tpl == 1 && s.rpl == 1 && s.sym == 0 && s.cl == 0 &&
+           s.persist == 0 && s.f64 == 0 && s.bal == 0 && s.warps == 8 && s.chunk == 0 &&
+           max_lysosome(c) <= 512;
   if (s.sym) {  // symmetric form: (warps, cells per warp) of its field kernel
     if (!c->fp32 || s.rpl != 1 || s.tpl != 2 * s.sym || s.tile != 32) return false;
     if (!((s.warps == 4 && (s.sym == 1 || s.sym == 2)) || (s.warps == 8 && s.sym == 1) ||
@@ -1082,7 +1114,7 @@ float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
   a.cos_k = 1.0;
   a.S = 1;
   a.n_rec = 1;
-  if (s.persist) {  // a persistent launch of 32 steps, timed twice after one
+  if (s.persist || s.clu) {  // a launch of 32 steps, timed twice after one
     constexpr int kSteps = 32;
     if (prepare_persist(c, kSteps) != KMC_OK) return -1.f;
     cudaEvent_t e0, e1;
@@ -1091,9 +1123,12 @@ float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
       cudaEventDestroy(e0);
       return -1.f;
     }
-    bool ok = launch_period(c, a, s, kSteps) == cudaSuccess;
+    auto period = [&]() {
+      return s.clu ? launch_cluster(c, a, kSteps, true) : launch_period(c, a, s, kSteps);
+    };
+    bool ok = period() == cudaSuccess;
     if (ok) ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
-    for (int r = 0; r < 2 && ok; ++r) ok = launch_period(c, a, s, kSteps) == cudaSuccess;
+    for (int r = 0; r < 2 && ok; ++r) ok = period() == cudaSuccess;
     if (ok) ok = cudaEventRecord(e1, c->stream) == cudaSuccess;
     if (ok) ok = cudaEventSynchronize(e1) == cudaSuccess;
     float ms = -1.f;
@@ -1189,9 +1224,9 @@ kmc_status autotune(kmc_ctx *c) {
     if (!log) return;
     std::fprintf(stderr,
                  "kmc tune %s: warps %d tile %d chunk %d tpl %d rpl %d sym %d cl %d supd %d "
-                 "persist %d f64 %d bal %d: %.4f ms per step\n",
+                 "persist %d f64 %d bal %d clu %d: %.4f ms per step\n",
                  what, s.warps, s.tile, s.chunk, s.tpl, s.rpl, s.sym, s.cl, s.supd, s.persist,
-                 s.f64, s.bal, ms);
+                 s.f64, s.bal, s.clu, ms);
   };
   auto consider = [&](const Shape &s, float ms) {
     show("shape", s, ms);
@@ -1294,13 +1329,30 @@ kmc_status autotune(kmc_ctx *c) {
     s.f64 = parts;
     consider(s, time_shape(c, s));
   }
+  // the whole period in clusters (tests: KMC_TUNE_CLUSTER, wherever it can run)
+  bool clu_pin = false;
+  if (c->fp32 && max_n <= 512 && c->persist_mode == 0 && c->cl_mode != 2 && c->rpl_mode <= 1 &&
+      c->tpl_mode <= 1 && !sym_only) {
+    Shape s;
+    s.warps = 8;
+    s.tile = 64;
+    s.clu = 1;
+    consider(s, time_shape(c, s));
+    clu_pin = std::getenv("KMC_TUNE_CLUSTER") != nullptr && !timed.empty() &&
+              s == timed.back().second;
+    if (clu_pin) {
+      best = timed.back().first;
+      bs = s;
+      timed.assign(1, timed.back());
+    }
+  }
   const int warps_c[] = {4, 8};
   const int tiles_f32[] = {64, 128, 256, 512};
   const int tiles_f64[] = {32, 64, 128, 128};  // (the FP64 list has three distinct tiles)
   const int chunks[] = {0, 256, 512, 1024, 2048, 4096, 8192};
   // replicas per lane (FP32, sets of identical lysosomes): one or four warps
   // per replica, one target per lane, tiles of 32..128 records per replica
-  for (int rpl = 2; rpl <= 4 && c->fp32 && c->tpl_mode <= 1 && !sym_only; rpl += 2) {
+  for (int rpl = 2; rpl <= 4 && c->fp32 && c->tpl_mode <= 1 && !sym_only && !clu_pin; rpl += 2) {
     if (!c->rep_ok[rpl] || (c->rpl_mode != 0 && c->rpl_mode != rpl)) continue;
     for (int wpr : {1, 2, 4}) {
       for (int t : {32, 64, 128}) {
@@ -1320,7 +1372,7 @@ kmc_status autotune(kmc_ctx *c) {
     }
   }
   for (int w : warps_c) {
-    if (f64_pin > 0 && bs.f64 > 0) break;
+    if ((f64_pin > 0 && bs.f64 > 0) || clu_pin) break;
     if (c->rpl_mode > 1 || sym_only) break;  // pinned replicas or form: only their shapes
     for (int q = 0; q < (c->fp32 ? 4 : 3); ++q) {
       const int t = c->fp32 ? tiles_f32[q] : tiles_f64[q];
@@ -1954,19 +2006,20 @@ kmc_status kmc_run(kmc_ctx *c, const double *mu0Hmax, int32_t n_amp, double f, i
   RunState rs{c->step_global, 0, 0};
   KMC_CUDA(cudaMemcpyAsync(c->d_rs, &rs, sizeof(rs), cudaMemcpyHostToDevice, c->stream));
   const Shape &sh = c->shape;
-  if (sh.persist) {  // one persistent launch per period, then the period advance
+  const bool whole = sh.persist || sh.clu;
+  if (whole) {  // one launch per period, then the period advance
     StepArgs a = base_args(c);
     a.seed = seed;
     a.discard = discard;
     a.n_rec = static_cast<int>(std::max(n_rec, 1ll));
     KMC_TRY(prepare_persist(c, S));
     for (int p = 0; p < periods; ++p) {
-      KMC_CUDA(launch_period(c, a, sh, S));
+      KMC_CUDA(sh.clu ? launch_cluster(c, a, S, true) : launch_period(c, a, sh, S));
       KMC_CUDA(kmc::launch_advance(c->d_rs, S, c->stream));
     }
   }
   // otherwise one field period (S step launches + the period advance) as a CUDA graph
-  if (!sh.persist && (!c->gexec || c->g_S != S || c->g_discard != discard || c->g_nrec != n_rec ||
+  if (!whole && (!c->gexec || c->g_S != S || c->g_discard != discard || c->g_nrec != n_rec ||
       !(c->g_shape == sh) || c->g_seed != seed)) {
     drop_graph(c);
     StepArgs a = base_args(c);
@@ -1981,7 +2034,7 @@ kmc_status kmc_run(kmc_ctx *c, const double *mu0Hmax, int32_t n_amp, double f, i
     c->g_shape = sh;
     c->g_seed = seed;
   }
-  for (int p = 0; p < periods && !sh.persist; ++p)
+  for (int p = 0; p < periods && !whole; ++p)
     KMC_CUDA(cudaGraphLaunch(c->gexec, c->stream));
   c->step_global += static_cast<long long>(S) * periods;
   c->have_run = true;

@@ -34,6 +34,11 @@ cudaError_t launch_step(int prec_fp32, int warps, int tile, const StepArgs &a, i
 cudaError_t launch_persist(const StepArgs &a, int warps, int tile, int n_items, cudaStream_t st);
 cudaError_t persist_blocks_per_sm(int warps, int tile, int *blocks);
 
+// A whole period (a.S steps) of small lysosomes, one cluster of `blocks` blocks
+// per lysosome (FP32; blocks = ceil(max_n / 32) <= 16). Writes the moments, the
+// records of the run and the counters, not the source records in a.src.
+cudaError_t launch_cluster(const StepArgs &a, int blocks, int max_n, cudaStream_t st);
+
 // Symmetric pair form (FP32): one step = kmc_field_sym<warps, cells> over
 // a.sitems[0 .. n_field) and then kmc_update_sym over a.supd[0 .. a.n_upd).
 // (warps, cells) in {(2, 2), (4, 1), (4, 2), (8, 1)}; row groups of warps x cells

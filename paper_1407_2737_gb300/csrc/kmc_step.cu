@@ -2231,6 +2231,7 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32)
 
 }  // namespace kmc
 
+#include "kmc_cluster.cuh"
 #include "kmc_field_f64.cuh"
 
 namespace kmc {
@@ -2363,6 +2364,24 @@ cudaError_t launch_persist(const StepArgs &a, int warps, int tile, int n_items, 
   if (warps == 4) return cudaLaunchKernelEx(&cfg, kmc_persist_f32<4>, a, tile);
   if (warps == 8) return cudaLaunchKernelEx(&cfg, kmc_persist_f32<8>, a, tile);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_cluster(const StepArgs &a, int blocks, int max_n, cudaStream_t st) {
+  if (blocks < 1 || blocks > kClusterMaxBlocks || max_n > blocks * kTargets)
+    return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.n_lys * blocks));
+  cfg.blockDim = dim3(kClusterWarps * 32);
+  cfg.dynamicSmemBytes = cluster_smem(max_n);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(blocks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kmc_cluster_f32<kClusterWarps>, a, blocks);
 }
 
 // Symmetric form: the field kernel over n_field items, then the update kernel
@@ -2579,6 +2598,10 @@ cudaError_t init_device() {
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym<8>);
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym_block<4>);
   if (e == cudaSuccess) e = allow_smem(kmc_update_sym_block<8>);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kmc_cluster_f32<kClusterWarps>,
+                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = allow_smem(kmc_cluster_f32<kClusterWarps>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<4>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<8>);
   if (e == cudaSuccess) e = allow_smem(kmc_step_f64<16>);
