@@ -66,8 +66,9 @@ __global__ void __launch_bounds__(32) kmc_field_f64(const StepArgs a, int /*tile
   if (!f64_item_in_bounds(a, it)) return;
   const int lane = threadIdx.x;
   const bool diag = it.g == it.h;
+  const long long step = a.rs->step_base + a.k_local;  // before the wait, as in kmc_step_f32
   grid_dependency_wait();
-  const int par = static_cast<int>((a.rs->step_base + a.k_local) & 1);
+  const int par = static_cast<int>(step & 1);
   const dbl4 *__restrict__ pos = static_cast<const dbl4 *>(a.src_pos);
   const dbl4 *__restrict__ mu = static_cast<const dbl4 *>(a.src[par]);
   const F64Src t = f64_source(pos, mu, it.g + lane, lane < it.ng);
@@ -138,9 +139,11 @@ __global__ void __launch_bounds__(kF64UpdWarps * 32)
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char *dyn = smem + 16;
   __shared__ GridTables<double> tab;
-  tab.load();
   if (!KMC_DCHECK(static_cast<int>(blockIdx.x) < a.n_upd, a.err, kSiteItem)) return;
-  const F64Upd u = a.fupd[blockIdx.x];
+  const F64Upd u = a.fupd[blockIdx.x];  // read in kmc_update_sym's order
+  const long long step = a.rs->step_base + a.k_local;
+  const int per = a.rs->period;
+  tab.load();
   if (!KMC_DCHECK(u.l >= 0 && u.l < a.n_lys, a.err, kSiteLys)) return;
   const LysDev L = a.lys[u.l];
   if (!KMC_DCHECK(u.t0 == 32 * u.cell && u.nt >= 1 && u.nt <= 32 && u.t0 + u.nt <= L.n &&
@@ -158,8 +161,6 @@ __global__ void __launch_bounds__(kF64UpdWarps * 32)
   it.split = 0;
   it.nsplit = 1;
   grid_dependency_wait();
-  const long long step = a.rs->step_base + a.k_local;
-  const int per = a.rs->period;
   const int rec = (per >= a.discard) ? (per - a.discard) * a.S + a.k_local : -1;
   TargetIn<dbl4> tin;
   if (warp == 0) tin = load_target<dbl4>(a, L, it, step, lane);

@@ -1932,8 +1932,8 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nc = (L.n + kCell - 1) / kCell;
   const int cell0 = it.g * GC + warp * C;  // the warp's first target cell
+  const long long step = a.rs->step_base + a.k_local;  // before the wait, as in kmc_step_f32
   grid_dependency_wait();
-  const long long step = a.rs->step_base + a.k_local;
   const int par = static_cast<int>(step & 1);
   const SrcPair *__restrict__ gsrc = static_cast<const SrcPair *>(a.src[par]) + L.roff;
 
@@ -2080,6 +2080,33 @@ __global__ void __launch_bounds__(W * 32) kmc_field_sym(const StepArgs a, int /*
   grid_launch_dependents();
 }
 
+// Adds, with compensation, the three components of slots first, first + step, ...
+// below count to (hi, lo): slot s at base + s slot, component q at + q comp. The
+// loads of kBatch slots are issued before any is added, and slots past the end
+// count as zero: with a break instead of that predicate the compiler loaded them
+// one by one, and a target's 55 to 150 slots each waited for the L2 in turn
+// (9 200 cycles of an update block's 18 400 at 8000 NPs, now 2 300).
+template <int kBatch>
+__device__ __forceinline__ void gather_slots(const float *base, size_t slot, int comp, int first,
+                                             int step, int count, float (&hi)[3],
+                                             float (&lo)[3]) {
+#pragma unroll 1
+  for (int s0 = first; s0 < count; s0 += step * kBatch) {
+    float v[kBatch][3];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const bool in = s0 + b * step < count;
+      const float *p = base + (in ? s0 + b * step : s0) * slot;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) v[b][q] = in ? __ldcg(p + q * comp) : 0.f;
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) neumaier_add(hi[q], lo[q], v[b][q]);
+  }
+}
+
 template <int GC>
 __global__ void __launch_bounds__(kSymUpdWarps * 32) kmc_update_sym(const StepArgs a, int /*tile*/) {
   constexpr int NW = kSymUpdWarps;
@@ -2087,13 +2114,17 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32) kmc_update_sym(const StepAr
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char *dyn = smem + 16;
   __shared__ GridTables<float> tab;
-  tab.load();
-  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ui = blockIdx.x * NW + warp;  // this warp's update item
-  if (ui >= a.n_upd || !sym_upd_in_bounds(a, GC, ui)) return;
-  const SymUpd u = a.supd[ui];
+  // what the runs of a period share is read ahead of the wait (the run state too:
+  // kmc_step_f32), the item first: the lysosome's constants hang on it
+  const SymUpd u = a.supd[min(ui, a.n_upd - 1)];
+  const long long step = a.rs->step_base + a.k_local;
+  const int per = a.rs->period;
+  tab.load();
   const LysDev L = a.lys[u.l];
+  __syncthreads();
+  if (ui >= a.n_upd || !sym_upd_in_bounds(a, GC, ui)) return;
   Item it;
   it.l = u.l;
   it.t0 = u.t0;
@@ -2103,48 +2134,17 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32) kmc_update_sym(const StepAr
   it.split = 0;
   it.nsplit = 1;
   grid_dependency_wait();
-  const long long step = a.rs->step_base + a.k_local;
-  const int per = a.rs->period;
   const int rec = (per >= a.discard) ? (per - a.discard) * a.S + a.k_local : -1;
   const TargetIn<float4> tin = load_target<float4>(a, L, it, step, lane);
   // lanes past the last target repeat it (their results are not written)
   const int tl = min(lane, u.nt - 1);
   const int gi = u.gt0 + tl, ci = (u.t0 + tl) % kCell;
-  // the slots in order; each batch's loads are issued before its additions
+  // the slots in order
   float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f};
-  constexpr int kFwdBatch = 8, kRevBatch = 8;
-#pragma unroll 1
-  for (int s0 = 0; s0 < u.nfwd; s0 += kFwdBatch) {
-    float v[kFwdBatch][3];
-#pragma unroll
-    for (int b = 0; b < kFwdBatch; ++b) {
-      const float *p = a.sfwd + static_cast<size_t>(u.fwd0 + min(s0 + b, u.nfwd - 1)) * 3 * GT;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) v[b][q] = __ldcg(p + q * GT + gi);
-    }
-#pragma unroll
-    for (int b = 0; b < kFwdBatch; ++b) {
-      if (s0 + b >= u.nfwd) break;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) neumaier_add(hi[q], lo[q], v[b][q]);
-    }
-  }
-#pragma unroll 1
-  for (int s0 = 0; s0 < u.nrev; s0 += kRevBatch) {
-    float v[kRevBatch][3];
-#pragma unroll
-    for (int b = 0; b < kRevBatch; ++b) {
-      const float *p = a.srev + static_cast<size_t>(u.rev0 + min(s0 + b, u.nrev - 1)) * 3 * kCell;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) v[b][q] = __ldcg(p + q * kCell + ci);
-    }
-#pragma unroll
-    for (int b = 0; b < kRevBatch; ++b) {
-      if (s0 + b >= u.nrev) break;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) neumaier_add(hi[q], lo[q], v[b][q]);
-    }
-  }
+  gather_slots<8>(a.sfwd + static_cast<size_t>(u.fwd0) * 3 * GT + gi, 3 * GT, GT, 0, 1, u.nfwd,
+                  hi, lo);
+  gather_slots<8>(a.srev + static_cast<size_t>(u.rev0) * 3 * kCell + ci, 3 * kCell, kCell, 0, 1,
+                  u.nrev, hi, lo);
   EpiShared<float> &sm = reinterpret_cast<EpiShared<float> *>(dyn)[warp];
 #pragma unroll
   for (int q = 0; q < 3; ++q) sm.h[q][lane] = hi[q] + lo[q];  // compensation added last
@@ -2169,9 +2169,11 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32)
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char *dyn = smem + 16;
   __shared__ GridTables<float> tab;
-  tab.load();
   if (!sym_upd_in_bounds(a, GC, static_cast<int>(blockIdx.x))) return;
-  const SymUpd u = a.supd[blockIdx.x];
+  const SymUpd u = a.supd[blockIdx.x];  // read in kmc_update_sym's order
+  const long long step = a.rs->step_base + a.k_local;
+  const int per = a.rs->period;
+  tab.load();
   const LysDev L = a.lys[u.l];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   Item it;
@@ -2183,8 +2185,6 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32)
   it.split = 0;
   it.nsplit = 1;
   grid_dependency_wait();
-  const long long step = a.rs->step_base + a.k_local;
-  const int per = a.rs->period;
   const int rec = (per >= a.discard) ? (per - a.discard) * a.S + a.k_local : -1;
   TargetIn<float4> tin;
   if (warp == 0) tin = load_target<float4>(a, L, it, step, lane);
@@ -2192,18 +2192,10 @@ __global__ void __launch_bounds__(kSymUpdWarps * 32)
   const int tl = min(lane, u.nt - 1);
   const int gi = u.gt0 + tl, ci = (u.t0 + tl) % kCell;
   float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f};
-#pragma unroll 1
-  for (int sl = warp; sl < u.nfwd; sl += NW) {
-    const float *p = a.sfwd + static_cast<size_t>(u.fwd0 + sl) * 3 * GT;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) neumaier_add(hi[q], lo[q], __ldcg(p + q * GT + gi));
-  }
-#pragma unroll 1
-  for (int sl = warp; sl < u.nrev; sl += NW) {
-    const float *p = a.srev + static_cast<size_t>(u.rev0 + sl) * 3 * kCell;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) neumaier_add(hi[q], lo[q], __ldcg(p + q * kCell + ci));
-  }
+  gather_slots<7>(a.sfwd + static_cast<size_t>(u.fwd0) * 3 * GT + gi, 3 * GT, GT, warp, NW,
+                  u.nfwd, hi, lo);
+  gather_slots<7>(a.srev + static_cast<size_t>(u.rev0) * 3 * kCell + ci, 3 * kCell, kCell, warp,
+                  NW, u.nrev, hi, lo);
   float *wp = reinterpret_cast<float *>(dyn);  // [NW][6][32]
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
