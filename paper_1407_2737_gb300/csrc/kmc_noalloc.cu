@@ -47,6 +47,11 @@ constexpr int kMaxSplit = 16;                                   // source ranges
 constexpr int kMaxItems = 1024;                                 // blocks
 constexpr int kTile = 128;                                      // records per staged tile
 constexpr int kWarps = 4;
+// Up to kOneMaxN NPs a block takes 32 targets, one per lane, and all sources: more
+// blocks and nothing to hand over. Pack and field kernels, two targets per lane in
+// ranges against this: 100 NPs 6.0 against 5.6 us, 200 7.3 against 6.5, 333 7.7 against
+// 7.4, 450 7.7 against 7.75, 600 7.9 against 8.7 (8 or 16 warps: the same or slower).
+constexpr int kOneMaxN = 448;
 constexpr size_t kRecBytes = sizeof(SrcPair) * kMaxRec;
 constexpr size_t kTgtBytes = sizeof(float4) * kMaxN;
 constexpr size_t kPartBytes = sizeof(float) * 6 * kGroup * kMaxItems;  // (sum, error) x 3
@@ -120,29 +125,31 @@ __global__ void noalloc_pack(unsigned char *scratch, int n, const double *__rest
   sc_tgt(scratch)[i] = make_float4(x, y, z, w);
 }
 
-// The records of one staged tile taken by this warp (every kWarps-th) against
-// the lane's two targets.
-template <bool MASK>
+// The records of one staged tile taken by this warp (every NW-th) against the
+// lane's TPL targets.
+template <bool MASK, int TPL, int NW>
 __device__ __forceinline__ void tile_pairs(const ulonglong2 *__restrict__ sp, int cnt, int first,
-                                           const f2 (&X)[2], const f2 (&Y)[2], const f2 (&Z)[2],
-                                           AccF32 (&acc)[2]) {
+                                           const f2 (&X)[TPL], const f2 (&Y)[TPL],
+                                           const f2 (&Z)[TPL], AccF32 (&acc)[TPL]) {
 #pragma unroll 8
-  for (int r = first; r < cnt; r += kWarps) {
+  for (int r = first; r < cnt; r += NW) {
     ulonglong2 a, b, c, d;
     f2 e;
     kmc::load_record(sp, r, a, b, c, d, e);
-    kmc::pair_record<MASK>(a, b, c, d, e, X[0], Y[0], Z[0], acc[0]);
-    kmc::pair_record<MASK>(a, b, c, d, e, X[1], Y[1], Z[1], acc[1]);
+#pragma unroll
+    for (int k = 0; k < TPL; ++k)
+      kmc::pair_record<MASK>(a, b, c, d, e, X[k], Y[k], Z[k], acc[k]);
   }
 }
 
 // Source ranges per group for G groups and nrec source records. Rough cycles:
-// an SM works a block's range off at 22.5 per record (64 targets, 18 packed
-// instructions per record and target at 0.8 of the pipe) plus 600; a block alone on
+// an SM works a block's range off at 20 per record (64 targets, 18 packed
+// instructions per record and target at 0.9 of the pipe) plus 1000; a block alone on
 // its SM takes 27 per record (one warp per scheduler) plus 2000 for its first
-// tile and epilogue; handing partial sums over costs 1500, and 30 for each. The
-// minimum over the ranges that the scratch holds fills the SMs where there are
-// few groups and evens out the last wave where there are many.
+// tile and epilogue; handing partial sums over costs 800, 60 for each and 600 for
+// the second batch of eight loads. The minimum over the ranges that the scratch holds
+// fills the SMs where there are few groups and evens out the last wave where there
+// are many: over 450 .. 8192 NPs it is within 3 % of the best range count measured.
 int splits_for(int G, int nrec) {
   constexpr int kSms = 152;
   int best = 1;
@@ -151,9 +158,9 @@ int splits_for(int G, int nrec) {
     const double r = static_cast<double>(nrec) / s;
     if (s > 1 && r < 16.0) break;
     const double per_sm = (G * s + kSms - 1) / kSms;
-    double t = per_sm * (22.5 * r + 600.0);
+    double t = per_sm * (20.0 * r + 1000.0);
     if (27.0 * r + 2000.0 > t) t = 27.0 * r + 2000.0;
-    if (s > 1) t += 1500.0 + 30.0 * s;
+    if (s > 1) t += 800.0 + 60.0 * s + (s > 8 ? 600.0 : 0.0);
     if (s == 1 || t < t_best) {
       best = s;
       t_best = t;
@@ -162,7 +169,7 @@ int splits_for(int G, int nrec) {
   return best;
 }
 
-// One block = 64 targets (two per lane: each staged record feeds two chains) x
+// One block = 32 TPL targets (two per lane: each staged record feeds two chains) x
 // one source range; the last block of a target group adds the partial sums in
 // split order and writes mu0 H_dip = bunit * b_dip, and the last group to finish
 // writes the status. A staging wait that runs out (after wait_ns) sets the error
@@ -171,34 +178,37 @@ int splits_for(int G, int nrec) {
 // that path) makes every tile expect that many bytes more than its copy
 // delivers, so that every wait runs out while no copy is left unfinished. Bound:
 // the FP32 pipe, as kmc_step_f32_tn, whose pair loop this is.
-// 8192 NPs: 52 us (7 ranges, 896 blocks) against 58 for one target per lane in ranges
-// of 512 records, the call 57 against 65; 3000 NPs 18.6 against 23.6 us.
-__global__ void __launch_bounds__(kWarps * 32, 4)
+// Pack and field kernels at 8192 NPs: 50.9 us (7 ranges, 896 blocks) against 60.0 for
+// one target per lane in ranges of 512 records; 3000 NPs 14.2 against 17.9 us, 1000
+// 8.5 against 13.8.
+template <int TPL, int NW>
+__global__ void __launch_bounds__(NW * 32, 16 / NW)
     noalloc_field(unsigned char *scratch, int n, int nsplit, double bunit,
                   double *__restrict__ B, int32_t *__restrict__ status, uint32_t stall_tx,
                   unsigned long long wait_ns) {
   __shared__ __align__(128) ulonglong2 buf[2][kTile * kmc::kRecU2];
-  __shared__ float wp[kWarps][12][32];
+  __shared__ float wp[NW][6 * TPL][32];
   __shared__ uint64_t bar[2];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
-  const int t0 = kGroup * g, nt = min(kGroup, n - t0);
+  constexpr int kTargets = 32 * TPL;  // of the block
+  const int t0 = kTargets * g, nt = min(kTargets, n - t0);
   const int nrec = (n + 1) / 2;
   const int j0 = static_cast<int>(static_cast<long long>(split) * nrec / nsplit);
   const int j1 = static_cast<int>(static_cast<long long>(split + 1) * nrec / nsplit);
   const int own0 = t0 >> 1, own1 = (t0 + nt - 1) >> 1;
-  f2 X[2], Y[2], Z[2];
+  f2 X[TPL], Y[TPL], Z[TPL];
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {  // lanes past the last target repeat it
+  for (int k = 0; k < TPL; ++k) {  // lanes past the last target repeat it
     const float4 p = sc_tgt(scratch)[t0 + min(32 * k + lane, nt - 1)];
     X[k] = kmc::pk(p.x, p.x);
     Y[k] = kmc::pk(p.y, p.y);
     Z[k] = kmc::pk(p.z, p.z);
   }
-  float s6[6], c6[6];
+  float s6[3 * TPL], c6[3 * TPL];
 #pragma unroll
-  for (int c = 0; c < 6; ++c) s6[c] = c6[c] = 0.f;
+  for (int c = 0; c < 3 * TPL; ++c) s6[c] = c6[c] = 0.f;
   const SrcPair *src = sc_rec(scratch);
   int32_t *err = sc_err(scratch);
   const int ntiles = (j1 - j0 + kTile - 1) / kTile;
@@ -223,15 +233,15 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
     const bool ok = kmc::mbar_wait_bounded(&bar[t & 1], (t >> 1) & 1, err, wait_ns);
     if (ok) {
       const int r0 = j0 + t * kTile, cnt = min(kTile, j1 - r0);
-      AccF32 acc[2];
+      AccF32 acc[TPL];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) acc[k].x = acc[k].y = acc[k].z = 0ull;
+      for (int k = 0; k < TPL; ++k) acc[k].x = acc[k].y = acc[k].z = 0ull;
       if (r0 <= own1 && own0 < r0 + cnt)
-        tile_pairs<true>(buf[t & 1], cnt, warp, X, Y, Z, acc);
+        tile_pairs<true, TPL, NW>(buf[t & 1], cnt, warp, X, Y, Z, acc);
       else
-        tile_pairs<false>(buf[t & 1], cnt, warp, X, Y, Z, acc);
+        tile_pairs<false, TPL, NW>(buf[t & 1], cnt, warp, X, Y, Z, acc);
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < TPL; ++k) {
         kmc::kahan_add(s6[3 * k + 0], c6[3 * k + 0], kmc::hsum(acc[k].x));
         kmc::kahan_add(s6[3 * k + 1], c6[3 * k + 1], kmc::hsum(acc[k].y));
         kmc::kahan_add(s6[3 * k + 2], c6[3 * k + 2], kmc::hsum(acc[k].z));
@@ -249,31 +259,31 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
   }
   if (failed) {
 #pragma unroll
-    for (int c = 0; c < 6; ++c) s6[c] = __int_as_float(0x7fc00000);  // NaN
+    for (int c = 0; c < 3 * TPL; ++c) s6[c] = __int_as_float(0x7fc00000);  // NaN
   }
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
+  for (int c = 0; c < 3 * TPL; ++c) {
     wp[warp][c][lane] = s6[c];
-    wp[warp][6 + c][lane] = -c6[c];
+    wp[warp][3 * TPL + c][lane] = -c6[c];
   }
   __syncthreads();
-  // warp k < 2: the lane's target 32 k + lane
+  // warp k < TPL: the lane's target 32 k + lane
   float hi[3], lo[3];
-  if (warp < 2) {
+  if (warp < TPL) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       float s = 0.f, e = 0.f;
-      for (int w = 0; w < kWarps; ++w) {
+      for (int w = 0; w < NW; ++w) {
         kmc::neumaier_add(s, e, wp[w][3 * warp + c][lane]);
-        e += wp[w][6 + 3 * warp + c][lane];
+        e += wp[w][3 * TPL + 3 * warp + c][lane];
       }
       hi[c] = s;
       lo[c] = e;
     }
   }
   if (nsplit > 1) {
-    constexpr size_t kItem = 6 * kGroup;  // floats: [2 parts][6][32]
-    if (warp < 2) {
+    constexpr size_t kItem = 6 * kTargets;  // floats: [TPL parts][6][32]
+    if (warp < TPL) {
       float *part = sc_part(scratch) + blockIdx.x * kItem + warp * 192;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -282,29 +292,37 @@ __global__ void __launch_bounds__(kWarps * 32, 4)
       }
     }
     if (!kmc::arrive_last(&sc_cnt(scratch)[g], nsplit, &s_last)) return;
-    if (warp < 2) {
-      const float *base = sc_part(scratch) + (blockIdx.x - split) * kItem + warp * 192;
+    if (warp < TPL) {
+      // the ranges in order, the loads of eight at a time issued before their sums (ranges
+      // past the last add zeros: with a break the loads go out one by one)
+      const float *base = sc_part(scratch) + (blockIdx.x - split) * kItem + warp * 192 + lane;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        float s = 0.f, e = 0.f;
-#pragma unroll 4
-        for (int q = 0; q < nsplit; ++q) {
-          kmc::neumaier_add(s, e, __ldcg(base + q * kItem + c * 32 + lane));
-          e += __ldcg(base + q * kItem + (3 + c) * 32 + lane);
-        }
-        hi[c] = s;
-        lo[c] = e;
+      for (int c = 0; c < 3; ++c) hi[c] = lo[c] = 0.f;
+      for (int q0 = 0; q0 < nsplit; q0 += 8) {
+        float v[8][6];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+          for (int c = 0; c < 6; ++c)
+            v[q][c] = q0 + q < nsplit ? __ldcg(base + (q0 + q) * kItem + c * 32) : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            kmc::neumaier_add(hi[c], lo[c], v[q][c]);
+            lo[c] += v[q][3 + c];
+          }
       }
     }
   }
   const int t = 32 * warp + lane;
-  if (warp < 2 && t < nt) {
+  if (warp < TPL && t < nt) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) B[3 * (t0 + t) + c] = bunit * static_cast<double>(hi[c] + lo[c]);
   }
   // the call's status once every group is done: KMC_OK, or KMC_ETIMEOUT if a wait ran out
   if (status && threadIdx.x == 0) {
-    const int groups = (n + kGroup - 1) / kGroup;
+    const int groups = (n + kTargets - 1) / kTargets;
     int32_t done;
     asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
                  : "=r"(done)
@@ -449,8 +467,12 @@ kmc_status kmc_dipolar_field_noalloc(int32_t n, const double *pos, const double 
                                                       center[1], center[2], inv_len, w_scale);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(KMC_ECUDA, "packing kernel launch failed", e);
-  noalloc_field<<<groups * nsplit, kWarps * 32, 0, st>>>(scratch, n, nsplit, kMu0 * Ms, B, status,
-                                                         stall_tx, wait_ns);
+  if (n <= kOneMaxN)
+    noalloc_field<1, kWarps><<<(n + 31) / 32, kWarps * 32, 0, st>>>(
+        scratch, n, 1, kMu0 * Ms, B, status, stall_tx, wait_ns);
+  else
+    noalloc_field<2, kWarps><<<groups * nsplit, kWarps * 32, 0, st>>>(
+        scratch, n, nsplit, kMu0 * Ms, B, status, stall_tx, wait_ns);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(KMC_ECUDA, "field kernel launch failed", e);
   return KMC_OK;

@@ -1,6 +1,6 @@
-"""kmc_dipolar_field_noalloc at the edges of its groups of 64 targets (two per
-lane) and of the source ranges that it cuts by size: one and two groups, ragged
-second targets, odd counts, ranges of a few records, the largest number of blocks.
+"""kmc_dipolar_field_noalloc at the edges of its groups of 32 (up to 448 NPs) and 64
+targets (two per lane) and of the source ranges that it cuts by size: one and two
+groups, ragged second targets, odd counts, ranges of a few records, the largest number of blocks.
 Tolerance: the FP32 field's, 1e-5 of the rms field, as in the other tests. The
 outputs of every NP are checked, the values beyond them stay as they were."""
 import numpy as np
@@ -12,7 +12,7 @@ from paper_1407_2737_gb300 import inputs, kmc
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [2, 31, 33, 63, 64, 65, 97, 128, 129, 333, 600, 2047, 4097, 8191])
+@pytest.mark.parametrize("n", [2, 31, 33, 63, 64, 65, 97, 128, 129, 333, 448, 449, 600, 2047, 4097, 8191])
 def test_group_edges(n):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
