@@ -2357,7 +2357,8 @@ kmc_status kmc_local_concentration(kmc_ctx *c, int32_t lys, int32_t N, double *p
   if (!c->d_phigrid) {
     size_t need = 0;
     for (int x : c->n) need = std::max(need, kmc::local_concentration_scratch(x));
-    if (need) KMC_TRY(dalloc(reinterpret_cast<char **>(&c->d_phigrid), need));
+    // (no room: all pairs, which need none of it)
+    if (need) dalloc(reinterpret_cast<char **>(&c->d_phigrid), need);
   }
   // the box of the positions about the frame origin and their largest distance
   // from it, in units of L (with a little slack for the rounding of the device's
@@ -2517,7 +2518,7 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   // bounding them too
   const size_t per_step = static_cast<size_t>(N) * (kmc::kMeanFields * sizeof(double) +
                                                     sizeof(int32_t));
-  const int span = static_cast<int>(std::min<long long>(
+  int span = static_cast<int>(std::min<long long>(
       std::min(S, 65536), std::max<long long>(1, static_cast<long long>((64u << 20) / per_step))));
   kmc::MeanArgs a;
   kmc::MeanLysDev *d_lys = nullptr;
@@ -2526,7 +2527,11 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   double *d_beta = nullptr, *d_vfrac = nullptr, *d_cos = nullptr;
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) {
-      KMC_TRY(dalloc(&sc.p, sc.used));
+      if (dalloc(&sc.p, sc.used) != KMC_OK) {
+        if (span == 1) return KMC_ENOMEM;
+        span /= 2;  // add up again for fewer steps at once
+        pass = 0;
+      }
       sc.used = 0;
     }
     sc.take(&d_lys, n_lys);

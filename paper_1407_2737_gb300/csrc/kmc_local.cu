@@ -20,9 +20,9 @@
 // ms; 200 NPs 70 against 445 us, so it serves all but the smallest sizes. At 50 000
 // and N = 64 0.59 ms against 266.
 //
-// All pairs (fewer NPs; NPs so unevenly spread that a cell holds more than
-// kPhiMaxCell; coordinates outside FP32's range): one thread per target keeps the
-// N smallest squared FP64 distances seen so far in ascending order. FP32 copies of
+// All pairs (fewer NPs; no device memory for the grid; NPs so unevenly spread that
+// a cell holds more than kPhiMaxCell; coordinates outside FP32's range): one thread
+// per target keeps the N smallest squared FP64 distances seen so far in ascending order. FP32 copies of
 // the source positions are staged through shared memory tile by tile, and an
 // FP32 pre-screen skips a pair whose FP32 squared distance exceeds the current
 // N-th by more than a bound on the FP32 error.
@@ -439,7 +439,7 @@ cudaError_t launch_local_concentration(const dbl4 *pos, int n, int N, double rma
   if (n <= 0) return cudaSuccess;
   PhiGrid g;
   const int *max_cell = nullptr;
-  if (n >= kPhiGridMin && n <= (1 << 28) && phi_grid(n, N, rmax, lo, hi, &g)) {
+  if (scratch && n >= kPhiGridMin && n <= (1 << 28) && phi_grid(n, N, rmax, lo, hi, &g)) {
     float4 *sorted = static_cast<float4 *>(scratch);
     const int padded = phi_padded_cells(g.nx * g.ny * g.nz);
     int *start = reinterpret_cast<int *>(sorted + n);  // 16-byte aligned
