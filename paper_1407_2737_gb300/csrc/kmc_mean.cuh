@@ -28,7 +28,7 @@
 // the nodes within its error (SignProfile) and Newton starts from an FP32 root
 // (root_in_cell). 2000 NPs, 200 steps: 75.4 ms with one
 // thread per NP for the whole run (63 warps on 152 SMs, every step a serial chain
-// of about 1.7e4 FP64 instructions), 0.85 ms now, of which the wells take 0.29 ms
+// of about 1.7e4 FP64 instructions), 0.75 ms now, of which the wells take 0.29 ms
 // and the carry 0.18 ms.
 #pragma once
 

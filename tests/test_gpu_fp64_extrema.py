@@ -73,16 +73,18 @@ def test_near_switching(eps):
         _check(_lone([math.pi - p], 2e4), h * (1 + eps) * 2 * 2e4 / MS)
 
 
-def test_mean_mode_in_spans():
-    # 10 000 NPs x 200 steps exceed the workspace, so the period is solved in
-    # several spans, anew in each period; the others fit and are solved once
-    big = inputs.lattice_nodes_lysosome(10000, 14e-9, 0.1, Keff=2e4, seed=1)
+@pytest.mark.parametrize("n,S,periods", [(10000, 200, 1), (10000, 200, 2), (40000, 400, 2)])
+def test_mean_mode_in_spans(n, S, periods):
+    # the first and the last exceed the workspace (64 MB; 1 GB for several periods), so
+    # a period is solved in spans, anew in each period; the others fit and are solved once
+    big = inputs.lattice_nodes_lysosome(n, 14e-9, 0.1, Keff=2e4, seed=1)
     small = inputs.lattice_nodes_lysosome(33, 14e-9, 0.1, Keff=2e4, seed=2)
     one = _lone([1.0], 2e4, T=0.0)[0]
-    g = kmc.kmc_mean_run([small, big, one], 0.03, 1e5, 200, 2, 0)
-    assert np.array_equal(kmc.kmc_mean_run([small, one], 0.03, 1e5, 200, 2, 0), g[[0, 2]])
+    g = kmc.kmc_mean_run([small, big, one], 0.03, 1e5, S, periods, 0)
+    assert np.array_equal(kmc.kmc_mean_run([small, one], 0.03, 1e5, S, periods, 0), g[[0, 2]])
     for q, ly in ((0, small), (2, one)):
-        o = oracle.mean_run(ly.axis, ly.vol, ly.Ms, ly.Keff, ly.T, ly.tau0, 0.03, 1e5, 200, 2, 0)
+        o = oracle.mean_run(ly.axis, ly.vol, ly.Ms, ly.Keff, ly.T, ly.tau0, 0.03, 1e5, S, periods,
+                            0)
         np.testing.assert_allclose(g[q], o, rtol=0, atol=1e-12)
 
 
