@@ -156,7 +156,6 @@ def fp32_lane_ops_peak():
     """FP32 lane operations per second: SMs x lanes x maximum SM clock."""
     return SMS * FP32_LANES * SM_MAX_MHZ * 1e6
 SMS, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
-FP64_PEAK_TFLOPS = 1.25      # nominal GB300 FP64 (FMA = 2 flops)
 HBM_GBS = 6771.5             # measured copy bandwidth of this pool's GB300s
 
 
@@ -332,17 +331,19 @@ def run_row(args):
         line = {"metric": "pair distances/s, local concentration phi_N (Eq. 8, N = 10)",
                 "value": value, "unit": "pairs/s", "ms_per_step": 1e3 * t,
                 "dtype": "f64", "config": {"workload": CONFIGS["c4"][0], "row": "f1",
-                                           "step": "phi_N of all 50 000 NPs (all pairs)"},
-                "roofline": {"bound": "alu", "achieved": 8 * value / 1e12,
-                             "peak": fp32_peak_tflops(), "unit": "TFLOP/s",
-                             "frac": 8 * value / 1e12 / fp32_peak_tflops(), "traffic": None,
-                             "kernel": "local_concentration_kernel",
-                             "note": "an FP32 pre-screen per pair (8 flops), FP64 only for "
-                                     "the pairs that can enter the N-nearest list; one warp "
-                                     "per 32 targets leaves ~9 warps per SM (latency-bound)"},
+                                           "step": "phi_N of all 50 000 NPs (the value counts all "
+                                                   "pairs; a grid search forms the near ones)"},
+                "roofline": {"bound": "hbm", "achieved": 40 * n / t / 1e9, "peak": HBM_GBS,
+                             "unit": "GB/s", "frac": 40 * n / t / 1e9 / HBM_GBS,
+                             "traffic": None, "kernel": "phi_grid_kernel",
+                             "note": "40 B per NP (position in, phi out); the state is "
+                                     "L2-resident and the search, about 5 N candidates per "
+                                     "target and one warp each, is bound by instructions; the "
+                                     "timed call includes the copy of phi to the host"},
                 "e2e": {"value": pairs / (t + t_create), "unit": "pairs/s",
                         "h2d_bytes_per_step": n * 7 * 8, "d2h_bytes_per_step": n * 8},
-                "gpu_launches": args.steps,
+                # bin, scan, scatter, search, finish and the all-pairs kernel, which returns
+                "gpu_launches": 6 * args.steps,
                 "cpu_baseline": {"value": len(idx) * (n - 1) / tc, "unit": "pairs/s",
                                  "cores": 1, "kind": "oracle",
                                  "sample": "phi_N of %d NPs against all %d (%.1f s)" % (
@@ -381,10 +382,8 @@ def run_row(args):
         used = []
         t = events(lambda k: used.append(kmc.kmc_regenerate_rsa(ctx, 0, R, d, 11, k + 1)))
         value = n / t
-        # distance checks: each candidate against the spheres kept before it,
-        # about used * n / 2, at 8 flops each (an FP32 pre-screen; FP64 only
-        # within the rounding margin around d)
-        flops = 8.0 * used[-1] * n / 2
+        # a centre per candidate; 120 B per NP for the arrays that follow, as in f2
+        gbs = (24.0 * used[-1] + 120.0 * n) / t / 1e9
         (l1,), _ = inputs.config_single2000(replicas=1, seed=0)
         R1 = inputs.lysosome_radius(l1.n, 14e-9, 0.10)
         t0 = time.perf_counter()
@@ -398,19 +397,19 @@ def run_row(args):
                 "config": {"workload": CONFIGS["c4"][0], "row": "f2r",
                            "step": "all 50 000 NPs placed anew (%d candidates), then the NP "
                                    "arrays rebuilt" % used[-1]},
-                "roofline": {"bound": "alu", "achieved": flops / t / 1e12,
-                             "peak": fp32_peak_tflops(), "unit": "TFLOP/s",
-                             "frac": flops / t / 1e12 / fp32_peak_tflops(), "traffic": None,
-                             "kernel": "rsa_check_kernel",
-                             "note": "8 FP32 flops per distance check, used * n / 2 checks; "
-                                     "sequential by definition: batches of candidates checked "
-                                     "in parallel, then kept in order by one thread, whose walk "
-                                     "and the per-batch launches bound the placement"},
+                "roofline": {"bound": "hbm", "achieved": gbs, "peak": HBM_GBS, "unit": "GB/s",
+                             "frac": gbs / HBM_GBS, "traffic": None,
+                             "kernel": "rsa_resolve_kernel",
+                             "note": "24 B per candidate and 120 B per NP; sequential by "
+                                     "definition: batches of candidates are checked in cell "
+                                     "lists in parallel and resolved in rounds by one block; "
+                                     "the rounds, the per-batch wait and the host copies bound "
+                                     "the placement"},
                 "e2e": {"value": value, "unit": "NPs/s", "h2d_bytes_per_step": n * 24,
                         "d2h_bytes_per_step": n * 24},
-                # batches of 2048 candidates, three kernels each; then the regeneration
+                # batches of 32 768 candidates, four kernels each; then the regeneration
                 # kernel and the two source refreshes
-                "gpu_launches": args.steps * (3 * -(-used[-1] // 2048) + 3),
+                "gpu_launches": args.steps * (4 * -(-used[-1] // 32768) + 3),
                 "cpu_baseline": {"value": l1.n / tc, "unit": "NPs/s", "cores": 1,
                                  "kind": "oracle",
                                  "sample": "the 2000-NP lysosome (cost grows as n^2), "
@@ -429,7 +428,9 @@ def run_row(args):
                 times.append(time.perf_counter() - t0)
         t = sum(times) / len(times)
         value = n_np * steps / t
-        flops = 1000  # the 200-node scan alone: 200 x (2 FMA + 1 MUL) in FP64
+        # the 200-node scan alone, 200 x (2 FMA + 1 MUL) in FP32, of every NP and step of
+        # a period (the period's wells serve all periods)
+        flops = 1000.0 * n_np * run["S"]
         t0 = time.perf_counter()
         l0 = lyss[0]
         oracle.mean_run(l0.axis, l0.vol, l0.Ms, l0.Keff, l0.T, l0.tau0, run["mu0Hmax"], run["f"],
@@ -439,18 +440,18 @@ def run_row(args):
                 "value": value, "unit": "particle-steps/s", "ms_per_step": 1e3 * t,
                 "dtype": "f64", "config": {"workload": WORKLOAD, "row": "f4",
                                            "step": "one whole mean-mode run of the workload"},
-                "roofline": {"bound": "alu", "achieved": flops * value / 1e12,
-                             "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                             "frac": flops * value / 1e12 / FP64_PEAK_TFLOPS, "traffic": None,
-                             "kernel": "kmc_mean_kernel",
-                             "note": "algorithmic flops count the 200-node scan only (1000 per "
-                                     "NP-step); one thread per NP runs the whole run and the "
-                                     "FP64 pipe is ~80 % busy with the Newton steps' FP64 "
-                                     "divisions, the exponentials and the sines (ncu)"},
+                "roofline": {"bound": "alu", "achieved": flops / t / 1e12,
+                             "peak": fp32_peak_tflops(), "unit": "TFLOP/s",
+                             "frac": flops / t / 1e12 / fp32_peak_tflops(), "traffic": None,
+                             "kernel": "kmc_mean_carry",
+                             "note": "algorithmic flops count the 200-node scan of one period "
+                                     "only; the carry, a chain of FP64 operations from each "
+                                     "step's occupations to the next, takes most of the time"},
                 "e2e": {"value": value, "unit": "particle-steps/s",
                         "h2d_bytes_per_step": n_np * 5 * 8, "d2h_bytes_per_step":
                         8 * len(lyss) * run["S"] * (run["periods"] - run["discard"])},
-                "gpu_launches": args.steps,
+                # the wells of the period, and the carry of each period
+                "gpu_launches": (1 + run["periods"]) * args.steps,
                 "cpu_baseline": {"value": l0.n * run["S"] * 2 / tc, "unit": "particle-steps/s",
                                  "cores": 1, "kind": "oracle",
                                  "sample": "2 periods of one 2000-NP lysosome (%.1f s)" % tc}}
