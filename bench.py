@@ -133,8 +133,10 @@ def launch_info(kmc, ctx, lyss):
                 ops += 14 * 2 * (gc * cell) * ((h1 - h0) * cell)
         chains = len(cut) - 1
         block = kmc.kmc_sym_update(ctx) == 2
-        launch.update({"pair_form": "symmetric", "chains": chains, "field_items": len(items),
-                       "update_items": len(upd), "update": "block" if block else "warp"})
+        launch.update({"pair_form": "symmetric", "chains": chains, "update_items": len(upd),
+                       "update": "block" if block else "warp"})
+        if chunk:  # 0: whole rows or balanced items
+            launch["field_items"] = len(items)
         return {"launch": launch, "kernel": "kmc_field_sym<%d, %d> + kmc_update_sym%s<%d>" % (
                     warps, cells, "_block" if block else "", gc),
                 "lane_ops_per_pair": ops / pairs, "chains": chains,
@@ -145,6 +147,13 @@ def launch_info(kmc, ctx, lyss):
         return {"launch": launch, "kernel": "kmc_persist_f32<%d>" % warps,
                 "lane_ops_per_pair": lane_ops_per_pair(rpl), "chains": 1,
                 "launches_per_period": lambda S: 1, "key": (warps, tile, chunk, tpl, rpl, "persist")}
+    if max(n) <= 512 and (warps, tile, chunk, tpl, rpl) == (8, 64, 0, 1, 1):
+        # the shape of a period in clusters (kmc_step_f32<8> can have it too: the count is
+        # the smaller of the two)
+        launch.update({"pair_form": "ordered", "chains": 1, "cluster_period": True})
+        return {"launch": launch, "kernel": "kmc_cluster_f32<8>",
+                "lane_ops_per_pair": lane_ops_per_pair(rpl), "chains": 1,
+                "launches_per_period": lambda S: 1, "key": (warps, tile, chunk, tpl, rpl, "cluster")}
     chains = min(len(lyss) // max(rpl, 1), kmc.KMC_MAX_CHAINS)
     launch.update({"pair_form": "ordered", "chains": chains})
     return {"launch": launch, "kernel": step_kernel(warps, tpl, rpl),
@@ -813,11 +822,12 @@ def main():
         kmc.kmc_sync(c64)
         t64 = e0.elapsed_time(e1) / 1e3
         w64, tl64, ch64 = kmc.kmc_tuning(c64)
+        form64 = "symmetric" if kmc.kmc_pair_form(c64) == kmc.FORM_SYMMETRIC else "ordered"
         units64 = n_np * S64 * per64
         fp64 = {"value": units64 / t64, "unit": UNIT,
                 "ms_per_step": 1e3 * t64 * units_per_step / units64,
                 "speedup_fp32_mixed": float(value / world / (units64 / t64)),
-                "launch": {"warps": w64, "tile": tl64, "chunk": ch64}}
+                "launch": {"warps": w64, "tile": tl64, "chunk": ch64, "pair_form": form64}}
         if not fp64_steps:
             sar64 = [kmc.kmc_read(c64, kmc.KMC_READ_SAR, l)[0] for l in range(len(lyss))]
             rel = abs(np.mean(sar32) - np.mean(sar64)) / abs(np.mean(sar64))

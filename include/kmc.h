@@ -241,12 +241,15 @@ kmc_status kmc_replicas_per_lane(kmc_ctx *ctx, int32_t rpl, int32_t *rpl_out);
  *     order and runs steps iii-vii (two launches per step and chain). The
  *     fields differ from the ordered form's by rounding only; results are
  *     deterministic and do not depend on the chaining.
- * form: 0 lets the autotuner choose (the default: it times both forms on
- * FP32 contexts), 1 or 2 pins one (2: KMC_EINVAL on FP64 contexts, with
+ * form: 0 lets the autotuner choose (the default: it times both forms, on FP64
+ * contexts too, whose symmetric form has kernels of its own and takes no pins),
+ * 1 or 2 pins one (2: KMC_EINVAL on FP64 contexts, with
  * replicas per lane pinned, or with 1 or 3 targets per lane pinned). A pinned
  * symmetric form reads kmc_tuning's warps (4; 8 with 2 targets per lane; 2
  * with 4) and chunk (source NPs per field item, a multiple of 64; 0 = all cells above
- * the row group); its tile is 32. The form in use (0 before the first
+ * the row group; the autotuner also times items of equal pair counts that start
+ * and end inside a cell, for which kmc_tuning reports chunk 0); its tile is 32. The
+ * form in use (0 before the first
  * tuning) is returned through form_out (may be NULL); form = -1 only reads it. */
 kmc_status kmc_pair_form(kmc_ctx *ctx, int32_t form, int32_t *form_out);
 
@@ -261,7 +264,9 @@ kmc_status kmc_pair_form(kmc_ctx *ctx, int32_t form, int32_t *form_out);
  * every work item's block resident at once; a plan with more items fails with
  * KMC_EINVAL. The results are the bits of the per-step launches at the same
  * warps (4 or 8), tile and chunk. mode: 0 lets the autotuner choose (the
- * default: it times both where the plan fits), 1 off, 2 on (KMC_EINVAL on FP64
+ * default: it times both where the plan fits, and for lysosomes of up to 512
+ * NPs also a period as one launch of thread-block clusters, one per lysosome,
+ * which is reported as off here), 1 off, 2 on (KMC_EINVAL on FP64
  * contexts). The value in use (0 before the first tuning) is returned through
  * mode_out (may be NULL); mode = -1 only reads it. */
 kmc_status kmc_persistent(kmc_ctx *ctx, int32_t mode, int32_t *mode_out);
@@ -358,8 +363,9 @@ kmc_status kmc_plan_items(const int32_t *n, int32_t n_lys, kmc_precision prec, i
 
 /* Eq. 8 (Sec. III.5): the local volume concentration around each NP of
  * lysosome `lys`, phi_N,i = 3 N V_i / (4 pi r_N^3) with r_N the distance from
- * NP i to its N-th nearest neighbour in the lysosome. Computed on the device
- * over all pairs in FP64; 1 <= N <= min(n - 1, KMC_PHI_MAX_N), else
+ * NP i to its N-th nearest neighbour in the lysosome. Computed on the device,
+ * r_N from FP64 distances (a grid search, or all pairs of small or very
+ * uneven samples: the same bits); 1 <= N <= min(n - 1, KMC_PHI_MAX_N), else
  * KMC_EINVAL. Writes phi[n] (host buffer of capacity cap; KMC_ECAPACITY and
  * *written = n if too small). Synchronises the context's stream. */
 kmc_status kmc_local_concentration(kmc_ctx *ctx, int32_t lys, int32_t N, double *phi,
@@ -387,7 +393,7 @@ kmc_status kmc_shell_profile(kmc_ctx *ctx, int32_t lys, double radius, int32_t n
  * probability of an old well goes to the new minimum whose basin contains it,
  * and Eqs. 3-5 relax the two occupations towards equilibrium over each step.
  * Arguments as kmc_create (positions are not used) and kmc_run, without a
- * seed; runs in FP64 on the device, one thread per NP. Writes the
+ * seed; runs on the device, the occupations and wells in FP64. Writes the
  * volume-weighted mean m_z after each recorded step of every lysosome,
  * loop_M [n_lys][S * (periods - discard)] (host buffer of capacity cap;
  * KMC_ECAPACITY and *written = the size needed if too small). Starts from

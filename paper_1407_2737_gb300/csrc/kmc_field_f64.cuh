@@ -21,8 +21,8 @@
 // instructions per ordered pair. Every item writes its sums to its own slot, and
 // the update adds a target's slots in a fixed order: results are deterministic
 // and do not depend on the batch. Per step against the ordered
-// kernel at its best shape: 100 NPs 18.5 against 36 us (parts 2, 4, 8, 16: 35.1,
-// 25.7, 21.2, 20.4), 400: 26 against 62, 1000: 54 against 73, 2000: 152 against 214,
+// kernel at its best shape: 100 NPs 17.2 against 36 us (parts 2, 4, 8, 16: 35.0,
+// 25.3, 20.8, 19.4 when timed), 400: 26 against 62, 1000: 54 against 73, 2000: 150 against 214,
 // 4000: 523 against 754, where the pipe is 88 % busy. The autotuner times both.
 #pragma once
 

@@ -57,7 +57,8 @@ cudaError_t sym_blocks_per_sm(int warps, int cells, int *blocks);
 cudaError_t step_blocks_per_sm(int prec_fp32, int warps, int tile, int tpl, int *blocks,
                                int rpl = 1);
 
-// The Ref. [8] mode over all items of a (one warp per item).
+// The Ref. [8] mode over all items of a (32 NPs per item): wells, then carry, per
+// span of steps.
 cudaError_t launch_mean(const MeanArgs &a, cudaStream_t st);
 
 // Redraws the axes and/or positions of one lysosome (a.off .. a.off + a.n).
