@@ -2515,7 +2515,7 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   KMC_CUDA(cudaStreamCreateWithFlags(&b.st, cudaStreamNonBlocking));
   const size_t nl = static_cast<size_t>(std::max(need, 1ll));
   // steps solved at once: a period where 1 GB holds it and it serves several periods
-  // (16 000 NPs, 20 periods of 200 steps: 48.9 -> 7.5 ms a call), else as many as 64 MB hold (at
+  // (16 000 NPs, 20 periods of 200 steps: 48.9 -> 5.8 ms a call), else as many as 64 MB hold (at
   // least one), the launch's grid bounding them too
   const size_t per_step = static_cast<size_t>(N) * (kmc::kMeanFields * sizeof(double) +
                                                     sizeof(int32_t));

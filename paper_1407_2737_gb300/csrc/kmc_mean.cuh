@@ -28,8 +28,8 @@
 // the nodes within its error (SignProfile) and Newton starts from an FP32 root
 // (root_in_cell). 2000 NPs, 200 steps: 75.4 ms with one
 // thread per NP for the whole run (63 warps on 152 SMs, every step a serial chain
-// of about 1.7e4 FP64 instructions), 0.75 ms now, of which the wells take 0.29 ms
-// and the carry 0.18 ms.
+// of about 1.7e4 FP64 instructions), 0.65 ms now, of which the wells take 0.29 ms
+// and the carry 0.09 ms.
 #pragma once
 
 namespace kmc {
@@ -173,14 +173,26 @@ __global__ void __launch_bounds__(kMeanWarps * 32)
   }
 }
 
+// on_arc by FP32 angles (all within 1e-6 rad of the FP64 ones) unless x lies within
+// 1e-5 rad of an end. The ends are maxima of different brackets, 0.03 rad apart at least.
+__device__ __forceinline__ bool on_arc_fast(double x, double from, double to) {
+  const float t = static_cast<float>(x), f = static_cast<float>(from), e = static_cast<float>(to);
+  const float d1 = fabsf(t - f), d2 = fabsf(t - e);
+  const float near = fminf(fminf(d1, Prec<float>::two_pi - d1), fminf(d2, Prec<float>::two_pi - d2));
+  return near > 1e-5f ? on_arc<float>(t, f, e) : on_arc<double>(x, from, to);
+}
+
 // One block per item of 32 NPs: the probabilities through steps k0 .. k1 - 1 of
 // period p, from and to the state of the NPs (a.state; first: the start of the
 // run), in tiles of kCarryTile steps. Warp 0 runs the chain of a tile, which is
-// all that is serial (occupations of a step from those before it); meanwhile the
-// other warps load the next tile's wells into shared memory and reduce the
-// previous tile's contributions to the loop. One warp doing all three took 242 us
-// for 200 steps of 2000 NPs. Now 180 us.
-constexpr int kCarryTile = 8, kCarryHelpers = 4;
+// all that is serial: occupations of a step from those before it, four dependent
+// FP64 operations. Meanwhile the helper warps, one per step of a tile, load the
+// next tile into shared memory, find for its steps which basin holds the wells of
+// the step before (on_arc_fast; a span's first step and one that follows a step
+// without wells are left to the chain) and reduce the previous tile's
+// contributions to the loop. 200 steps of 2000 NPs: one warp doing all of it 242 us, with
+// four helpers and the basins in the chain 182, now 87.
+constexpr int kCarryTile = 8, kCarryHelpers = 8;
 
 __global__ void __launch_bounds__(32 * (1 + kCarryHelpers))
     kmc_mean_carry(const MeanArgs a, int k0, int k1, int p, int first) {
@@ -193,7 +205,7 @@ __global__ void __launch_bounds__(32 * (1 + kCarryHelpers))
   const bool active = lane < it.nt;
   const int i = L.off + it.t0 + min(lane, it.nt - 1);
   const int steps = k1 - k0, tiles = (steps + kCarryTile - 1) / kCarryTile;
-  // helpers: the wells of tile t, the steps in turn
+  // helpers: the wells of tile t, and where those of the step before went
   auto load = [&](int t) {
     for (int q = warp - 1; q < kCarryTile; q += kCarryHelpers) {
       const int r = t * kCarryTile + q;
@@ -202,7 +214,20 @@ __global__ void __launch_bounds__(32 * (1 + kCarryHelpers))
       double v[kMeanFields];
 #pragma unroll
       for (int f = 0; f < kMeanFields; ++f) v[f] = src[static_cast<size_t>(f) * a.n];
-      const int flag = a.flags[static_cast<size_t>(r) * a.n + i];
+      int flag = a.flags[static_cast<size_t>(r) * a.n + i];
+      double t0 = 0.0, t1 = 0.0;
+      int before = 0;
+      if (r > 0) {
+        t0 = src[-static_cast<long long>(kMeanFields) * a.n];
+        t1 = src[-static_cast<long long>(kMeanFields) * a.n + a.n];
+        before = a.flags[static_cast<size_t>(r - 1) * a.n + i];
+      }
+      if ((flag & 3) == 2 && (before & 3) != 0 && !(before & kMeanSkip)) {
+        const bool arcA = (flag & kMeanArc) != 0;
+        flag |= kMeanKnown;
+        if (on_arc_fast(t0, v[2], v[3]) == arcA) flag |= kMeanIn0;
+        if (on_arc_fast(t1, v[2], v[3]) == arcA) flag |= kMeanIn1;
+      }
 #pragma unroll
       for (int f = 0; f < kMeanFields; ++f) s_well[t & 1][q][f][lane] = v[f];
       s_flag[t & 1][q][lane] = flag;
@@ -262,10 +287,14 @@ __global__ void __launch_bounds__(32 * (1 + kCarryHelpers))
           p0 = 1.0;
           p1 = 0.0;
         } else if (nmin == 2) {
-          const double M1 = w[2][lane], M2 = w[3][lane], pinf = w[4][lane];
-          const bool arcA = (flag & kMeanArc) != 0;
-          const bool in0 = on_arc<double>(th0, M1, M2) == arcA;
-          const bool in1 = on_arc<double>(th1, M1, M2) == arcA;
+          const double pinf = w[4][lane];
+          bool in0 = (flag & kMeanIn0) != 0, in1 = (flag & kMeanIn1) != 0;
+          if (!(flag & kMeanKnown)) {
+            const double M1 = w[2][lane], M2 = w[3][lane];
+            const bool arcA = (flag & kMeanArc) != 0;
+            in0 = on_arc<double>(th0, M1, M2) == arcA;
+            in1 = on_arc<double>(th1, M1, M2) == arcA;
+          }
           double pA = (in0 ? p0 : 0.0) + (in1 ? p1 : 0.0);
           double pB = (in0 ? 0.0 : p0) + (in1 ? 0.0 : p1);
           if (flag & kMeanRelax) {

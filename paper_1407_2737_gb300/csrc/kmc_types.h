@@ -260,6 +260,9 @@ enum : int32_t {
   kMeanArc = 4,    // the first minimum lies on the arc from the first maximum to the second
   kMeanRelax = 8,  // the occupations relax (T > 0 and a rate above 0)
   kMeanSkip = 16,  // more than two minima or maxima: the step is skipped, an error set
+  // kmc_mean_carry's own: the step before had wells too, and which of them lie in the
+  // basin of this step's first minimum
+  kMeanKnown = 32, kMeanIn0 = 64, kMeanIn1 = 128,
 };
 
 // Sample regeneration between loops (kmc_regen.cuh), one lysosome per launch.
