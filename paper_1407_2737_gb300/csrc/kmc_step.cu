@@ -619,11 +619,12 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
       P = 0.0;
       if (!exact_p) {
         // relative error of Pf below 1.2e-6: 2 ulp in each exponential, then
-        // the sum, the quotient, expm1 and the product; a NaN (overflow) is not settled
+        // the sum, the quotient, expm1 and the product. Where a rate or their sum
+        // exceeds FP32 the quotient is 0 or a NaN: not settled
         const float ea = exp_fp64_arg(xa), eb = exp_fp64_arg(xb), sum = ea + eb;
         const float Pf = (sum > 0.f) ? (ea / sum) * (-expm1f(-sum)) : 0.f;
         const float uf = static_cast<float>(u);
-        settled = fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
+        settled = isfinite(sum) && fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
         P = Pf;
       }
       if (!settled) {
