@@ -453,6 +453,10 @@ kmc_status kmc_regenerate_rsa(kmc_ctx *ctx, int32_t lys, double radius, double d
  * if the call had not been made). KMC_EINVAL on an FP32 context. */
 kmc_status kmc_debug_stall(kmc_ctx *ctx);
 
+/* A test of the paths without room, on the host: with the environment variable
+ * KMC_FAULT=alloc_over:<bytes> every device allocation of a context or a call
+ * that is larger is refused as if the device were full. */
+
 /* Frees the context and its device memory. NULL-safe. */
 void kmc_destroy(kmc_ctx *ctx);
 

@@ -302,9 +302,18 @@ struct kmc_ctx {
 
 namespace {
 
+// Test of the paths without room (kmc.h): KMC_FAULT=alloc_over:<bytes> refuses
+// larger device allocations.
+bool alloc_refused(size_t bytes) {
+  const char *fault = std::getenv("KMC_FAULT");
+  return fault && std::strncmp(fault, "alloc_over:", 11) == 0 &&
+         bytes > std::strtoull(fault + 11, nullptr, 10);
+}
+
 template <typename T>
 kmc_status dalloc(T **p, size_t bytes) {
-  if (cudaMalloc(reinterpret_cast<void **>(p), bytes ? bytes : 16) != cudaSuccess) {
+  if (alloc_refused(bytes) ||
+      cudaMalloc(reinterpret_cast<void **>(p), bytes ? bytes : 16) != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
     return fail(KMC_ENOMEM, "cudaMalloc of %zu bytes failed", bytes);
@@ -850,6 +859,7 @@ StepArgs base_args(kmc_ctx *c) {
 // per-step launches of a period graph receive) and its barrier counters.
 kmc_status prepare_persist(kmc_ctx *c, int steps) {
   if (c->cosk_steps == steps) return KMC_OK;
+  c->cosk_steps = 0;  // until the table and the counters are whole
   if (!c->d_gbar) KMC_TRY(dalloc(&c->d_gbar, 2 * sizeof(uint32_t)));
   if (static_cast<size_t>(steps) > c->cosk_cap) {
     if (c->d_cosk) cudaFree(c->d_cosk);
@@ -858,7 +868,6 @@ kmc_status prepare_persist(kmc_ctx *c, int steps) {
     KMC_TRY(dalloc(&c->d_cosk, sizeof(double) * steps));
     c->cosk_cap = static_cast<size_t>(steps);
   }
-  c->cosk_steps = 0;
   std::vector<double> cs(static_cast<size_t>(steps));
   for (int k = 0; k < steps; ++k) cs[k] = std::cos(2.0 * kPi * k / steps);
   KMC_CUDA(cudaMemcpyAsync(c->d_cosk, cs.data(), sizeof(double) * cs.size(),
@@ -870,6 +879,7 @@ kmc_status prepare_persist(kmc_ctx *c, int steps) {
 
 // One persistent launch of `steps` steps (the barrier counters zeroed first).
 cudaError_t launch_period(kmc_ctx *c, StepArgs a, const Shape &sh, int steps) {
+  if (!c->d_cosk || !c->d_gbar) return cudaErrorInvalidValue;
   a.S = steps;
   a.cosk = c->d_cosk;
   a.gbar = c->d_gbar;
@@ -888,6 +898,7 @@ int max_lysosome(const kmc_ctx *c) {
 // or, without, a.cos_k.
 cudaError_t launch_cluster(const kmc_ctx *c, StepArgs a, int steps, bool table) {
   const int n = max_lysosome(c);
+  if (table && !c->d_cosk) return cudaErrorInvalidValue;
   a.S = steps;
   a.cosk = table ? c->d_cosk : nullptr;
   return kmc::launch_cluster(a, (n + kmc::kTargets - 1) / kmc::kTargets, n, c->stream);
