@@ -171,8 +171,10 @@ kmc_status kmc_debug_step(kmc_ctx *ctx, const double *mu0Hext, double t_step,
 
 /* Checkpoint: writes the moments and the global step counter to `path`;
  * kmc_load restores them into a context built from the same lysosomes and
- * precision, so that the next kmc_run continues bit for bit. kmc_load
- * refuses, leaving the context as it was: a file that is not a checkpoint or
+ * precision, so that the next kmc_run continues bit for bit under the same
+ * launch shape (kmc_launch_shape reads it and sets it, in another process
+ * too: the autotuner's choice may differ from one process to the next).
+ * kmc_load refuses, leaving the context as it was: a file that is not a checkpoint or
  * is cut short (KMC_EIO), one of another context (KMC_EINVAL), or one holding
  * a moment that is not a finite unit vector (KMC_EINVAL). */
 kmc_status kmc_save(kmc_ctx *ctx, const char *path);
@@ -193,7 +195,8 @@ kmc_status kmc_info(const kmc_ctx *ctx, int64_t *n_total, int32_t *n_lys,
  * may be NULL); call with warps = tile = chunk = -1 to only read it. With the
  * environment variable KMC_TUNE_LOG set (and not "0") the autotuner prints
  * every shape it times, the finalists' second timings and its choice on
- * standard error. */
+ * standard error. kmc_launch_shape reads and sets whole shapes, with what the
+ * three numbers here do not tell. */
 kmc_status kmc_tuning(kmc_ctx *ctx, int32_t warps, int32_t tile, int32_t chunk,
                       int32_t *warps_out, int32_t *tile_out, int32_t *chunk_out);
 
@@ -242,14 +245,14 @@ kmc_status kmc_replicas_per_lane(kmc_ctx *ctx, int32_t rpl, int32_t *rpl_out);
  *     fields differ from the ordered form's by rounding only; results are
  *     deterministic and do not depend on the chaining.
  * form: 0 lets the autotuner choose (the default: it times both forms, on FP64
- * contexts too, whose symmetric form has kernels of its own and takes no pins),
- * 1 or 2 pins one (2: KMC_EINVAL on FP64 contexts, with
+ * contexts too, whose symmetric form has kernels of its own and is set by
+ * kmc_launch_shape alone), 1 or 2 pins one (2: KMC_EINVAL on FP64 contexts, with
  * replicas per lane pinned, or with 1 or 3 targets per lane pinned). A pinned
  * symmetric form reads kmc_tuning's warps (4; 8 with 2 targets per lane; 2
  * with 4) and chunk (source NPs per field item, a multiple of 64; 0 = all cells above
  * the row group; the autotuner also times items of equal pair counts that start
- * and end inside a cell, for which kmc_tuning reports chunk 0); its tile is 32. The
- * form in use (0 before the first
+ * and end inside a cell, for which kmc_tuning reports chunk 0 and which
+ * kmc_launch_shape sets); its tile is 32. The form in use (0 before the first
  * tuning) is returned through form_out (may be NULL); form = -1 only reads it. */
 kmc_status kmc_pair_form(kmc_ctx *ctx, int32_t form, int32_t *form_out);
 
@@ -266,7 +269,7 @@ kmc_status kmc_pair_form(kmc_ctx *ctx, int32_t form, int32_t *form_out);
  * warps (4 or 8), tile and chunk. mode: 0 lets the autotuner choose (the
  * default: it times both where the plan fits, and for lysosomes of up to 512
  * NPs also a period as one launch of thread-block clusters, one per lysosome,
- * which is reported as off here), 1 off, 2 on (KMC_EINVAL on FP64
+ * which is reported as off here and told and set by kmc_launch_shape), 1 off, 2 on (KMC_EINVAL on FP64
  * contexts). The value in use (0 before the first tuning) is returned through
  * mode_out (may be NULL); mode = -1 only reads it. */
 kmc_status kmc_persistent(kmc_ctx *ctx, int32_t mode, int32_t *mode_out);
@@ -305,6 +308,45 @@ kmc_status kmc_sym_update(kmc_ctx *ctx, int32_t mode, int32_t *mode_out);
  * KMC_EINVAL). The value in use (0 before the first tuning) is returned
  * through mode_out (may be NULL); mode = -1 only reads it. */
 kmc_status kmc_cluster_split(kmc_ctx *ctx, int32_t mode, int32_t *mode_out);
+
+/* Fields of a launch shape (kmc_launch_shape). */
+#define KMC_SHAPE_FIELDS 12
+enum {
+  KMC_SHAPE_WARPS = 0,          /* warps per block (kmc_tuning)               */
+  KMC_SHAPE_TILE = 1,           /* records per tile; 32 in the symmetric forms,
+                                   64 for a period in clusters                */
+  KMC_SHAPE_CHUNK = 2,          /* source NPs per item (0 = not split)        */
+  KMC_SHAPE_TPL = 3,            /* targets per lane, >= 1                     */
+  KMC_SHAPE_RPL = 4,            /* replicas per lane, 1 = off                 */
+  KMC_SHAPE_SYM_CELLS = 5,      /* FP32 symmetric form: cells per warp, 1 or 2
+                                   (targets per lane twice that); 0 = ordered */
+  KMC_SHAPE_SYM_UPDATE = 6,     /* its update: 0 = a warp per item, 1 = a block */
+  KMC_SHAPE_BALANCED = 7,       /* it has items of about equal work, this many
+                                   waves of the blocks that the SMs hold, at
+                                   most 64 (chunk 0); 0 = items of whole cells */
+  KMC_SHAPE_CLUSTER = 8,        /* 2 = cluster split (kmc_cluster_split), else 0 */
+  KMC_SHAPE_PERSISTENT = 9,     /* 1 = persistent period (kmc_persistent)     */
+  KMC_SHAPE_CLUSTER_PERIOD = 10,/* 1 = a period as one launch of clusters (FP32,
+                                   lysosomes of up to 512 NPs, warps 8, tile 64,
+                                   chunk 0, one target and replica per lane)  */
+  KMC_SHAPE_FP64_PARTS = 11     /* FP64 symmetric form: parts per pair of cells
+                                   of 32 NPs, 1, 2, 4, 8 or 16 (warps 4, tile
+                                   32, chunk 0), while its partial sums, 1.5 KB
+                                   per part, stay within 1 GB; 0 = ordered    */
+};
+
+/* The whole launch shape in one call: get (may be NULL) receives the shape in
+ * use (KMC_SHAPE_FIELDS values, all 0 before the first tuning), set (may be
+ * NULL) takes such values, so that a run can be repeated bit for bit by
+ * another context or process on the same kind of GPU. All of set 0, or its
+ * warps 0: the autotuner chooses on the next kmc_run or kmc_debug_step.
+ * KMC_EINVAL, with the shape left as it was, for values that no kernel of the
+ * context runs or that contradict a pinned choice. (A plan that cannot be
+ * built, as a cluster split of groups that are not in two parts, is refused
+ * by the run.) Tests make the autotuner take one of these kinds whatever its
+ * timing: the environment variables KMC_TUNE_F64=<parts>, KMC_TUNE_BAL=<waves>
+ * (the symmetric form's only plans then) and KMC_TUNE_CLUSTER=1. */
+kmc_status kmc_launch_shape(kmc_ctx *ctx, const int32_t *set, int32_t *get);
 
 /* Fields of one field item and of one update item in kmc_plan_sym's output. */
 #define KMC_SYM_FIELDS 8

@@ -661,6 +661,12 @@ long long f64_pairs(const kmc_ctx *c) {
   return n;
 }
 
+// Whether its partial sums (1.5 KB per item) stay within 1 GB.
+bool f64_fits(const kmc_ctx *c, int parts) {
+  return f64_pairs(c) * parts * kmc::kF64Slot * static_cast<long long>(sizeof(double)) <=
+         (1ll << 30);
+}
+
 // The FP64 symmetric form's plan, `parts` parts per cell pair: lysosomes
 // largest first, each as its cell pairs in order (their parts in order) and one
 // update item per cell; chains cut at lysosome boundaries as in plan_sym.
@@ -992,10 +998,11 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
     return false;
   if (s.clu != 0)
     return c->fp32 && s.clu == 1 && s.tpl == 1 && s.rpl == 1 && s.sym == 0 && s.cl == 0 &&
-           s.persist == 0 && s.f64 == 0 && s.bal == 0 && s.warps == 8 && s.chunk == 0 &&
-           max_lysosome(c) <= 512;
+           s.persist == 0 && s.f64 == 0 && s.bal == 0 && s.warps == 8 && s.tile == 64 &&
+           s.chunk == 0 && max_lysosome(c) <= 512;
   if (s.sym) {  // symmetric form: (warps, cells per warp) of its field kernel
-    if (!c->fp32 || s.rpl != 1 || s.tpl != 2 * s.sym || s.tile != 32) return false;
+    if (!c->fp32 || s.rpl != 1 || s.tpl != 2 * s.sym || s.tile != 32 || s.cl != 0 || s.f64 != 0)
+      return false;
     if (!((s.warps == 4 && (s.sym == 1 || s.sym == 2)) || (s.warps == 8 && s.sym == 1) ||
           (s.warps == 2 && s.sym == 2)))
       return false;
@@ -1005,7 +1012,8 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
   if (s.bal != 0) return false;
   if (s.f64 != 0)
     return !c->fp32 && s.tpl == 1 && s.rpl == 1 && s.cl == 0 && s.warps == 4 && s.tile == 32 &&
-           s.chunk == 0 && s.f64 > 0 && s.f64 <= 16 && (s.f64 & (s.f64 - 1)) == 0;
+           s.chunk == 0 && s.f64 > 0 && s.f64 <= 16 && (s.f64 & (s.f64 - 1)) == 0 &&
+           f64_fits(c, s.f64);
   if (s.tpl > 3) return false;
   if (s.cl != 0 && (s.cl != 2 || !c->fp32 || s.tpl != 1 || s.rpl != 1 || s.chunk <= 0))
     return false;
@@ -1020,6 +1028,19 @@ bool shape_ok(const kmc_ctx *c, const Shape &s) {
   if (s.warps != 4 && s.warps != 8 && s.warps != 16) return false;
   if (s.tile < 32 || s.tile > max_tile(c->fp32, s.warps) || (s.tile & (s.tile - 1))) return false;
   if (s.chunk < 0 || (s.chunk % 64) != 0) return false;
+  return true;
+}
+
+// Whether shape s keeps to the pinned choices that apply to its kind.
+bool pins_allow(const kmc_ctx *c, const Shape &s) {
+  const bool one = s.sym == 0 && s.tpl == 1 && s.rpl == 1;  // where cl and persist apply
+  if (c->tpl_mode != 0 && s.tpl != c->tpl_mode) return false;
+  if (c->rpl_mode != 0 && s.rpl != c->rpl_mode) return false;
+  if (c->form_mode != 0 && (s.sym != 0 || s.f64 != 0) != (c->form_mode == 2)) return false;
+  if (c->supd_mode != 0 && s.sym != 0 && s.supd != c->supd_mode - 1) return false;
+  if ((c->cl_mode == 1 && s.cl != 0) || (c->cl_mode == 2 && one && s.cl == 0)) return false;
+  if (c->persist_mode == 1 && (s.persist != 0 || s.clu != 0)) return false;
+  if (c->persist_mode == 2 && one && s.cl == 0 && s.persist == 0) return false;
   return true;
 }
 
@@ -1324,17 +1345,13 @@ kmc_status autotune(kmc_ctx *c) {
     }
   }
   // symmetric form in FP64: cell pairs cut in parts while the items are fewer
-  // than the warps that the SMs hold (32 blocks of one warp each, 152 SMs); its
-  // partial sums take 1.5 KB per item, at most 1 GB
+  // than the warps that the SMs hold (32 blocks of one warp each, 152 SMs)
   // (KMC_TUNE_F64=parts, for tests: that many parts, whatever the timings)
   const char *f64_env = c->fp32 ? nullptr : std::getenv("KMC_TUNE_F64");
   const int f64_pin = f64_env ? std::atoi(f64_env) : 0;
   for (int parts = 1; parts <= 16 && !c->fp32 && c->form_mode != 1; parts *= 2) {
-    const long long items = f64_pairs(c) * parts;
-    if (f64_pin > 0) {
-      if (parts != f64_pin) continue;
-    } else if ((parts > 1 && items > 32 * 152) ||
-        items * kmc::kF64Slot * static_cast<long long>(sizeof(double)) > (1ll << 30))
+    if (f64_pin > 0 && parts != f64_pin) continue;
+    if (!f64_fits(c, parts) || (f64_pin <= 0 && parts > 1 && f64_pairs(c) * parts > 32 * 152))
       break;
     Shape s;
     s.warps = 4;
@@ -1863,7 +1880,9 @@ kmc_status kmc_pair_form(kmc_ctx *c, int32_t form, int32_t *form_out) {
   if (form != -1) {
     if (form < 0 || form > 2)
       return fail(KMC_EINVAL, "pair form: 0 (autotuned), 1 (ordered) or 2 (symmetric)");
-    if (form == 2 && !c->fp32) return fail(KMC_EINVAL, "the symmetric form runs on FP32 contexts");
+    if (form == 2 && !c->fp32)
+      return fail(KMC_EINVAL, "FP64 contexts take their symmetric form from the autotuner or "
+                  "kmc_launch_shape");
     if (form == 2 && c->rpl_mode > 1)
       return fail(KMC_EINVAL, "the symmetric form does not run replicas per lane");
     if (form == 2 && (c->tpl_mode == 1 || c->tpl_mode == 3))
@@ -1971,6 +1990,56 @@ kmc_status kmc_tuning(kmc_ctx *c, int32_t warps, int32_t tile, int32_t chunk,
   if (warps_out) *warps_out = c->shape.warps;
   if (tile_out) *tile_out = c->shape.tile;
   if (chunk_out) *chunk_out = c->shape.chunk;
+  return KMC_OK;
+}
+
+kmc_status kmc_launch_shape(kmc_ctx *c, const int32_t *set, int32_t *get) {
+  if (!c) return fail(KMC_EINVAL, "ctx is NULL");
+  if (set && set[KMC_SHAPE_WARPS] == 0) {
+    c->shape = Shape();
+  } else if (set) {
+    // (the ranges of the fields that shape_ok takes for granted)
+    const int32_t rpl = set[KMC_SHAPE_RPL];
+    bool ok = set[KMC_SHAPE_TPL] >= 1 && set[KMC_SHAPE_TPL] <= 4 &&
+              (rpl == 1 || rpl == 2 || rpl == 4) && set[KMC_SHAPE_SYM_CELLS] >= 0 &&
+              set[KMC_SHAPE_SYM_CELLS] <= 2 && set[KMC_SHAPE_BALANCED] <= 64;
+    Shape s;
+    s.warps = set[KMC_SHAPE_WARPS];
+    s.tile = set[KMC_SHAPE_TILE];
+    s.chunk = set[KMC_SHAPE_CHUNK];
+    s.tpl = set[KMC_SHAPE_TPL];
+    s.rpl = rpl;
+    s.sym = set[KMC_SHAPE_SYM_CELLS];
+    s.supd = set[KMC_SHAPE_SYM_UPDATE];
+    s.bal = set[KMC_SHAPE_BALANCED];
+    s.cl = set[KMC_SHAPE_CLUSTER];
+    s.persist = set[KMC_SHAPE_PERSISTENT];
+    s.clu = set[KMC_SHAPE_CLUSTER_PERIOD];
+    s.f64 = set[KMC_SHAPE_FP64_PARTS];
+    if (!ok || !shape_ok(c, s))
+      return fail(KMC_EINVAL, "not a launch shape of this context (kmc_launch_shape)");
+    if (!pins_allow(c, s))
+      return fail(KMC_EINVAL, "the launch shape contradicts a pinned choice");
+    c->shape = s;
+  }
+  if (get) {
+    const Shape &s = c->shape;
+    std::memset(get, 0, sizeof(int32_t) * KMC_SHAPE_FIELDS);
+    if (s.warps != 0) {
+      get[KMC_SHAPE_WARPS] = s.warps;
+      get[KMC_SHAPE_TILE] = s.tile;
+      get[KMC_SHAPE_CHUNK] = s.chunk;
+      get[KMC_SHAPE_TPL] = s.tpl;
+      get[KMC_SHAPE_RPL] = s.rpl;
+      get[KMC_SHAPE_SYM_CELLS] = s.sym;
+      get[KMC_SHAPE_SYM_UPDATE] = s.supd;
+      get[KMC_SHAPE_BALANCED] = s.bal;
+      get[KMC_SHAPE_CLUSTER] = s.cl;
+      get[KMC_SHAPE_PERSISTENT] = s.persist;
+      get[KMC_SHAPE_CLUSTER_PERIOD] = s.clu;
+      get[KMC_SHAPE_FP64_PARTS] = s.f64;
+    }
+  }
   return KMC_OK;
 }
 

@@ -36,11 +36,14 @@ EXPORTS = ("kmc_create", "kmc_set_stream", "kmc_run", "kmc_read", "kmc_sync",
            "kmc_shell_profile", "kmc_mean_run", "kmc_regenerate", "kmc_debug_stall",
            "kmc_regenerate_rsa", "kmc_targets_per_lane", "kmc_plan_items",
            "kmc_replicas_per_lane", "kmc_pair_form", "kmc_plan_sym", "kmc_cluster_split",
-           "kmc_sym_update", "kmc_persistent", "kmc_debug_grid_stall")
+           "kmc_sym_update", "kmc_persistent", "kmc_debug_grid_stall", "kmc_launch_shape")
 KMC_NOALLOC_MAX_N = 8192
 KMC_MAX_CHAINS = 8  # parallel step-kernel chains of a batch (kmc_run)
 KMC_ITEM_FIELDS = 8  # per work item in kmc_plan_items
 KMC_SYM_FIELDS = 8  # per field and update item in kmc_plan_sym
+KMC_SHAPE_FIELDS = 12  # of a launch shape, in order (kmc_launch_shape):
+SHAPE_KEYS = ("warps", "tile", "chunk", "tpl", "rpl", "sym_cells", "sym_update", "balanced",
+              "cluster", "persistent", "cluster_period", "fp64_parts")
 KMC_CELL = 64  # NPs per cell of the symmetric pair form
 FORM_ORDERED, FORM_SYMMETRIC = 1, 2  # kmc_pair_form
 KMC_PHI_MAX_N = 64
@@ -110,6 +113,7 @@ def lib():
             L.kmc_sym_update.argtypes = [vp, C.c_int32, _I32]
             L.kmc_persistent.argtypes = [vp, C.c_int32, _I32]
             L.kmc_debug_grid_stall.argtypes = [vp]
+            L.kmc_launch_shape.argtypes = [vp, _I32, _I32]
             L.kmc_plan_sym.argtypes = [_I32, C.c_int32, C.c_int32, C.c_int32, _I32, C.c_int64,
                                        _I64, _I32, C.c_int64, _I64, _I64, _I32, _I32, _I32]
             L.kmc_plan_items.argtypes = [_I32, C.c_int32, C.c_int, C.c_int32, C.c_int32,
@@ -414,6 +418,16 @@ def kmc_tuning(ctx, warps=None, tile=None, chunk=0):
         _check(lib().kmc_tuning(ctx.handle, int(warps), int(tile), int(chunk), C.byref(w),
                                 C.byref(t), C.byref(c)))
     return int(w.value), int(t.value), int(c.value)
+
+
+def kmc_launch_shape(ctx, shape=None):
+    """The whole launch shape in use as a dict of SHAPE_KEYS (all 0 before the first
+    tuning); shape, such a dict, sets it first (warps 0: autotuned)."""
+    get = (C.c_int32 * KMC_SHAPE_FIELDS)()
+    new = None if shape is None else (C.c_int32 * KMC_SHAPE_FIELDS)(
+        *[int(shape[k]) for k in SHAPE_KEYS])
+    _check(lib().kmc_launch_shape(ctx.handle, new, get))
+    return dict(zip(SHAPE_KEYS, [int(x) for x in get]))
 
 
 def kmc_dipolar_field_noalloc(n, pos_dev, m_dev, vol_dev, Ms, center, length, B_dev,
