@@ -269,7 +269,8 @@ kmc_status kmc_pair_form(kmc_ctx *ctx, int32_t form, int32_t *form_out);
  * warps (4 or 8), tile and chunk. mode: 0 lets the autotuner choose (the
  * default: it times both where the plan fits, and for lysosomes of up to 512
  * NPs also a period as one launch of thread-block clusters, one per lysosome,
- * which is reported as off here and told and set by kmc_launch_shape), 1 off, 2 on (KMC_EINVAL on FP64
+ * which is reported as off here and told and set by kmc_launch_shape), 1 off
+ * (neither of the two: a shape in clusters is dropped), 2 on (KMC_EINVAL on FP64
  * contexts). The value in use (0 before the first tuning) is returned through
  * mode_out (may be NULL); mode = -1 only reads it. */
 kmc_status kmc_persistent(kmc_ctx *ctx, int32_t mode, int32_t *mode_out);

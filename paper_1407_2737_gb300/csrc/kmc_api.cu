@@ -1910,7 +1910,8 @@ kmc_status kmc_persistent(kmc_ctx *c, int32_t mode, int32_t *mode_out) {
     if (mode != 0 && c->shape.warps != 0) {
       Shape s = c->shape;
       s.persist = mode == 2 ? 1 : 0;
-      c->shape = shape_ok(c, s) ? s : Shape();
+      // (a period in clusters is one launch too: pinned off, the next run tunes anew)
+      c->shape = s.clu == 0 && shape_ok(c, s) ? s : Shape();
     }
   }
   if (mode_out)

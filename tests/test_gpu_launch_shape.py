@@ -124,3 +124,16 @@ def test_shapes_keep_to_the_pins():
         assert e.value.status == kmc.KMC_EINVAL
         kmc.kmc_launch_shape(ctx, _shape(**good))
         kmc.kmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_a_pinned_period_drops_the_clusters(mode):
+    # in either order: pinned before tuning, the mode keeps the cluster period out
+    ly = inputs.make_lysosome(90, 12e-9, 0.05, seed=3)
+    ctx = kmc.kmc_create([ly], F32, center=np.zeros(3))
+    kmc.kmc_launch_shape(ctx, _shape(**CLU))
+    kmc.kmc_persistent(ctx, mode)
+    kmc.kmc_run(ctx, 0.02, 1e5, 10, 1, 0, 5)
+    s = kmc.kmc_launch_shape(ctx)
+    assert s["cluster_period"] == 0 and (s["persistent"] == 0 or mode == 2)
+    kmc.kmc_destroy(ctx)
