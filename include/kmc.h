@@ -30,7 +30,8 @@
  *   - Device memory is allocated by kmc_create and freed by kmc_destroy.
  *   - Work is queued on the context's CUDA stream (a private stream unless
  *     kmc_set_stream gave one); kmc_run returns once the work is queued.
- *     kmc_read, kmc_sync, kmc_debug_step and kmc_save wait for it, and report
+ *     kmc_read, kmc_sync, kmc_debug_step and kmc_save wait for it (and for what
+ *     a caller has queued on a stream of its own before), and report
  *     KMC_ETIMEOUT if a device-side wait ran out of time.
  *   - A context is not thread-safe; distinct contexts are independent.
  */

@@ -953,11 +953,18 @@ kmc_status refresh_sources(kmc_ctx *c, int par) {
   return KMC_OK;
 }
 
+// Waits for queued work. On a caller's stream that is the caller's too, which this
+// context cannot know of; on its own there is none left once it has settled.
+kmc_status wait_queued(kmc_ctx *c) {
+  if (!c->settled || c->stream != c->own_stream) KMC_CUDA(cudaStreamSynchronize(c->stream));
+  return KMC_OK;
+}
+
 // Waits for queued work and reports the device error word (once: the reads that
 // follow a run one after another then cost their own copy alone, 14 us a call
 // instead of 35).
 kmc_status check_device_error(kmc_ctx *c) {
-  if (c->settled) return KMC_OK;
+  if (c->settled) return wait_queued(c);
   int32_t ew[2] = {0, 0};
   KMC_CUDA(cudaMemcpyAsync(ew, c->d_err, sizeof(ew), cudaMemcpyDeviceToHost, c->stream));
   KMC_CUDA(cudaStreamSynchronize(c->stream));
@@ -2146,7 +2153,7 @@ kmc_status kmc_read(kmc_ctx *c, int32_t what, int32_t lys, double *buf, int64_t 
       what == KMC_READ_AXES) {
     // state, readable after a device error so that the caller can see what
     // happened (kmc_sync reports the error)
-    if (!c->settled) KMC_CUDA(cudaStreamSynchronize(c->stream));
+    KMC_TRY(wait_queued(c));
   } else {
     KMC_TRY(check_device_error(c));
   }
