@@ -53,6 +53,13 @@ kmc_status fail(kmc_status s, const char *fmt, ...) {
   return s;
 }
 
+// Keeps the thread's message over an attempt whose failure is worked around: it is
+// that of a call that failed, not of one that succeeded without what it tried.
+struct KeepError {
+  const std::string kept = g_last_error;
+  ~KeepError() { g_last_error = kept; }
+};
+
 #define KMC_CUDA(call)                                                              \
   do {                                                                              \
     cudaError_t e_ = (call);                                                        \
@@ -1148,6 +1155,7 @@ kmc_status capture_steps(kmc_ctx *c, const StepArgs &a, const Shape &sh, int ste
 // over `scale` times the usual number of steps. Returns milliseconds per step,
 // or a negative value on error.
 float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
+  const KeepError keep;
   if (set_items(c, s) != KMC_OK) return -1.f;
   StepArgs a = base_args(c);
   a.cos_k = 1.0;
@@ -2446,6 +2454,7 @@ kmc_status kmc_local_concentration(kmc_ctx *c, int32_t lys, int32_t N, double *p
     size_t need = 0;
     for (int x : c->n) need = std::max(need, kmc::local_concentration_scratch(x));
     // (no room: all pairs, which need none of it)
+    const KeepError keep;
     if (need) dalloc(reinterpret_cast<char **>(&c->d_phigrid), need);
   }
   // the box of the positions about the frame origin and their largest distance
@@ -2619,8 +2628,10 @@ kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu
   double *d_beta = nullptr, *d_vfrac = nullptr, *d_cos = nullptr;
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) {
+      const std::string before = g_last_error;
       if (dalloc(&sc.p, sc.used) != KMC_OK) {
         if (span == 1) return KMC_ENOMEM;
+        g_last_error = before;
         span /= 2;  // add up again for fewer steps at once
         pass = 0;
       }
