@@ -991,6 +991,18 @@ kmc_status check_device_error(kmc_ctx *c) {
   return KMC_OK;
 }
 
+// The mean positions (those given at creation) and the current ones on the device,
+// both or neither.
+kmc_status ensure_nodes(kmc_ctx *c) {
+  if (c->d_nodes && c->d_possi) return KMC_OK;
+  const size_t bytes = sizeof(double) * 3 * c->N;
+  if (!c->d_nodes) KMC_TRY(dalloc(&c->d_nodes, bytes));
+  if (!c->d_possi) KMC_TRY(dalloc(&c->d_possi, bytes));
+  KMC_CUDA(cudaMemcpy(c->d_nodes, c->pos_si.data(), bytes, cudaMemcpyHostToDevice));
+  KMC_CUDA(cudaMemcpy(c->d_possi, c->pos_si.data(), bytes, cudaMemcpyHostToDevice));
+  return KMC_OK;
+}
+
 kmc_status upload_lys(kmc_ctx *c) {
   KMC_CUDA(cudaMemcpyAsync(c->d_lys, c->h_lys.data(), sizeof(LysDev) * c->n_lys,
                            cudaMemcpyHostToDevice, c->stream));
@@ -2276,10 +2288,8 @@ kmc_status kmc_debug_step(kmc_ctx *c, const double *mu0Hext, double t_step, uint
     if (!is_finite(m_in[i])) return fail(KMC_EINVAL, "non-finite moment");
   KMC_TRY(ensure_shape(c));
   const long long N = c->N;
-  if (!c->d_dbg) {
-    KMC_TRY(dalloc(&c->d_dbg, sizeof(double) * N * 7));
-    KMC_TRY(dalloc(&c->d_dbg_flags, sizeof(int32_t) * N));
-  }
+  if (!c->d_dbg) KMC_TRY(dalloc(&c->d_dbg, sizeof(double) * N * 7));
+  if (!c->d_dbg_flags) KMC_TRY(dalloc(&c->d_dbg_flags, sizeof(int32_t) * N));
   HostBytes h_m(c->vbytes * N);
   for (long long i = 0; i < N; ++i) {
     if (c->fp32)
@@ -2701,14 +2711,7 @@ kmc_status kmc_regenerate_rsa(kmc_ctx *c, int32_t lys, double radius, double dia
   const int n = c->n[lys];
   const long long cap = max_candidates > 0 ? max_candidates : 1000ll * n;
   KMC_TRY(check_device_error(c));
-  if (!c->d_nodes) {  // the mean positions: those given at creation
-    KMC_TRY(dalloc(&c->d_nodes, sizeof(double) * 3 * c->N));
-    KMC_TRY(dalloc(&c->d_possi, sizeof(double) * 3 * c->N));
-    KMC_CUDA(cudaMemcpy(c->d_nodes, c->pos_si.data(), sizeof(double) * 3 * c->N,
-                        cudaMemcpyHostToDevice));
-    KMC_CUDA(cudaMemcpy(c->d_possi, c->pos_si.data(), sizeof(double) * 3 * c->N,
-                        cudaMemcpyHostToDevice));
-  }
+  KMC_TRY(ensure_nodes(c));
   const int B = static_cast<int>(
       std::min<long long>(kmc::kRsaMaxBatch, std::max<long long>(256, 2ll * n)));
   kmc::RsaArgs a;
@@ -2822,14 +2825,7 @@ kmc_status kmc_regenerate(kmc_ctx *c, int32_t lys, int32_t what, double disorder
   if ((what & KMC_REGEN_POSITIONS) && !(disorder >= 0 && is_finite(disorder)))
     return fail(KMC_EINVAL, "disorder must be finite and >= 0");
   KMC_TRY(check_device_error(c));
-  if (!c->d_nodes) {  // the mean positions: those given at creation
-    KMC_TRY(dalloc(&c->d_nodes, sizeof(double) * 3 * c->N));
-    KMC_TRY(dalloc(&c->d_possi, sizeof(double) * 3 * c->N));
-    KMC_CUDA(cudaMemcpy(c->d_nodes, c->pos_si.data(), sizeof(double) * 3 * c->N,
-                        cudaMemcpyHostToDevice));
-    KMC_CUDA(cudaMemcpy(c->d_possi, c->pos_si.data(), sizeof(double) * 3 * c->N,
-                        cudaMemcpyHostToDevice));
-  }
+  KMC_TRY(ensure_nodes(c));
   const int l0 = lys < 0 ? 0 : lys, l1 = lys < 0 ? c->n_lys : lys + 1;
   for (int l = l0; l < l1; ++l) {
     kmc::RegenArgs a;
