@@ -469,7 +469,8 @@ __device__ __forceinline__ TargetState<R> setup_plane(R ax, R ay, R az, R mx, R 
 
 // Whether the projected moment lies on the arc from M1 to M2 (step v). FP64: the
 // FP32 angle decides (its error and the rounding of M1 and M2 to FP32 are below
-// 2e-6 rad) unless it lies within 1e-5 rad of either end.
+// 2e-6 rad) unless it lies within 1e-5 rad of either end, or the projection is so short
+// (a moment normal to the plane) that FP32 does not hold its direction.
 __device__ __forceinline__ bool moment_on_arc(const TargetState<float> &st, float M1, float M2) {
   return on_arc<float>(st.th0, M1, M2);
 }
@@ -479,7 +480,8 @@ __device__ __forceinline__ bool moment_on_arc(const TargetState<double> &st, dou
               m2 = static_cast<float>(M2);
   const float d1 = fabsf(t - m1), d2 = fabsf(t - m2);
   const float near = fminf(fminf(d1, Prec<float>::two_pi - d1), fminf(d2, Prec<float>::two_pi - d2));
-  if (near > 1e-5f) return on_arc<float>(t, m1, m2);
+  const float len = fmaxf(fabsf(static_cast<float>(st.m_a)), fabsf(static_cast<float>(st.m_e)));
+  if (near > 1e-5f && len > 1e-30f) return on_arc<float>(t, m1, m2);
   double th0 = atan2(st.m_e, st.m_a);
   if (th0 < 0.0) th0 += Prec<double>::two_pi;
   return on_arc<double>(th0, M1, M2);
