@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <new>
@@ -1165,15 +1166,21 @@ kmc_status capture_steps(kmc_ctx *c, const StepArgs &a, const Shape &sh, int ste
 
 // Times one candidate shape on the current state (restored by the caller),
 // over `scale` times the usual number of steps. Returns milliseconds per step,
-// or a negative value on error.
-float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
+// or a negative value on error. A candidate whose second launch alone took
+// longer than `hopeless` a step is given up with that time: most candidates are
+// 1.3 to 3 times slower than the best. First run of a size with all of them timed
+// in full and with this: 50 000 NPs 3.24 and 1.76 s, 96 lysosomes of about 1400
+// NPs 3.4 and 2.2 s, 8 x 2000 0.91 and 0.63 s, 8000 0.23 and 0.09 s, 1000 47 and
+// 45 ms, 100 7 and 4 ms.
+float time_shape(kmc_ctx *c, const Shape &s, float hopeless, int scale = 1) {
   const KeepError keep;
   if (set_items(c, s) != KMC_OK) return -1.f;
   StepArgs a = base_args(c);
   a.cos_k = 1.0;
   a.S = 1;
   a.n_rec = 1;
-  if (s.persist || s.clu) {  // a launch of 32 steps, timed twice after one
+  if (s.persist || s.clu) {  // a launch of 32 steps, timed twice after one (of one step
+                             // and a single one if that is hopeless)
     constexpr int kSteps = 32;
     if (prepare_persist(c, kSteps) != KMC_OK) return -1.f;
     cudaEvent_t e0, e1;
@@ -1182,16 +1189,22 @@ float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
       cudaEventDestroy(e0);
       return -1.f;
     }
-    auto period = [&]() {
-      return s.clu ? launch_cluster(c, a, kSteps, true) : launch_period(c, a, s, kSteps);
+    auto period = [&](int steps) {
+      return s.clu ? launch_cluster(c, a, steps, true) : launch_period(c, a, s, steps);
     };
-    bool ok = period() == cudaSuccess;
-    if (ok) ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
-    for (int r = 0; r < 2 && ok; ++r) ok = period() == cudaSuccess;
-    if (ok) ok = cudaEventRecord(e1, c->stream) == cudaSuccess;
-    if (ok) ok = cudaEventSynchronize(e1) == cudaSuccess;
     float ms = -1.f;
-    if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms /= 2 * kSteps;
+    // `reps` launches of 32 steps: milliseconds per step into ms
+    auto timed = [&](int reps) {
+      bool ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
+      for (int r = 0; r < reps && ok; ++r) ok = period(kSteps) == cudaSuccess;
+      if (ok) ok = cudaEventRecord(e1, c->stream) == cudaSuccess;
+      if (ok) ok = cudaEventSynchronize(e1) == cudaSuccess;
+      if (ok) ok = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+      ms /= reps * kSteps;
+      return ok;
+    };
+    bool ok = period(1) == cudaSuccess && timed(1);
+    if (ok && ms < hopeless) ok = timed(2);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaGetLastError();
@@ -1226,14 +1239,23 @@ float time_shape(kmc_ctx *c, const Shape &s, int scale = 1) {
     return launch_one_step(c, b, s, c->stream, true);
   };
   float ms = -1.f;
-  bool ok = true;
-  for (int r = 0; r < 2 && ok; ++r) ok = one() == cudaSuccess;
-  const int reps = (gx ? 2 : 5) * scale;
-  if (ok) ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
-  for (int r = 0; r < reps && ok; ++r) ok = one() == cudaSuccess;
-  if (ok) ok = cudaEventRecord(e1, c->stream) == cudaSuccess;
-  if (ok) ok = cudaEventSynchronize(e1) == cudaSuccess;
-  if (ok && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms /= reps * (gx ? graph_steps : 1);
+  // `reps` launches after `before` others: milliseconds per step into ms
+  auto timed = [&](int before, int reps) {
+    bool ok = true;
+    for (int r = 0; r < before && ok; ++r) ok = one() == cudaSuccess;
+    if (ok) ok = cudaEventRecord(e0, c->stream) == cudaSuccess;
+    for (int r = 0; r < reps && ok; ++r) ok = one() == cudaSuccess;
+    if (ok) ok = cudaEventRecord(e1, c->stream) == cudaSuccess;
+    if (ok) ok = cudaEventSynchronize(e1) == cudaSuccess;
+    if (ok) ok = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+    ms /= reps * (gx ? graph_steps : 1);
+    return ok;
+  };
+  // (the wait leaves the GPU idle: a single launch is led by an untimed one again)
+  const bool look = std::isfinite(hopeless);
+  bool ok = !look || timed(1, 1);
+  if (ok && (!look || ms < hopeless))
+    ok = timed(look ? (gx ? 0 : 1) : 2, (gx ? 2 : 5) * scale);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (gx) cudaGraphExecDestroy(gx);
@@ -1287,14 +1309,25 @@ kmc_status autotune(kmc_ctx *c) {
                  what, s.warps, s.tile, s.chunk, s.tpl, s.rpl, s.sym, s.cl, s.supd, s.persist,
                  s.f64, s.bal, s.clu, ms);
   };
-  auto consider = [&](const Shape &s, float ms) {
+  // Shapes are given up from 1.3 times the best so far on, or a likely one timed
+  // first: the chained launches of many steps, and single launches of 20 us and more,
+  // which an event pair times to a few per cent
+  float likely = 1e30f;
+  auto hopeless = [&](bool any = false) {
+    const float b = std::min(best, likely);
+    return b < 1e29f && (any || c->n_lys > 1 || b >= 0.02f)
+               ? 1.3f * b : std::numeric_limits<float>::infinity();
+  };
+  auto consider = [&](const Shape &s) {
+    const float ms = time_shape(c, s, hopeless());
     show("shape", s, ms);
-    if (!(ms > 0.f)) return;
+    if (!(ms > 0.f)) return ms;
     timed.emplace_back(ms, s);
     if (ms < best) {
       best = ms;
       bs = s;
     }
+    return ms;
   };
   bs.warps = 4;
   bs.tile = 64;
@@ -1311,6 +1344,20 @@ kmc_status autotune(kmc_ctx *c) {
     bs.tile = 32;
     bs.sym = c->tpl_mode == 4 ? 2 : 1;
     bs.tpl = 2 * bs.sym;
+  }
+  if (c->fp32 && c->form_mode == 0 && c->tpl_mode == 0 && c->rpl_mode <= 1 && c->cl_mode != 2 &&
+      c->persist_mode != 2) {
+    Shape s;
+    s.warps = 4;
+    s.tpl = 2;
+    s.tile = max_n < 3000 ? 64 : 32;
+    if (max_n >= 3000) {
+      s.sym = 2;
+      s.tpl = 4;
+      s.chunk = 512;
+    }
+    const float ms = time_shape(c, s, hopeless());
+    if (ms > 0.f) likely = ms;
   }
   // symmetric form (FP32): (warps, cells per warp), source NPs per field item
   const char *bal_env = std::getenv("KMC_TUNE_BAL");
@@ -1333,23 +1380,24 @@ kmc_status autotune(kmc_ctx *c) {
         s.tpl = 2 * v[1];
         s.sym = v[1];
         s.supd = c->supd_mode == 2 ? 1 : 0;
-        const float ms = time_shape(c, s);
-        consider(s, ms);
+        consider(s);
       }
-      // balanced items, 1, 2, 4 or 8 waves of them (tests: KMC_TUNE_BAL, only these)
+      // balanced items, 1, 2, 4 or 8 waves of them (tests: KMC_TUNE_BAL, only these), not
+      // where every pair lies inside a row group and the ordered form may run
       for (int bal : {1, 2, 4, 8}) {
-        if (bal_env && bal != std::atoi(bal_env)) continue;
+        if (bal_env ? bal != std::atoi(bal_env) : !sym_only && max_n <= gc * kmc::kCell) continue;
         Shape s;
         s.warps = v[0];
         s.tile = 32;
         s.tpl = 2 * v[1];
         s.sym = v[1];
         s.bal = bal;
-        // (their targets gather more slots, so both update kernels are timed)
+        // (their targets gather more slots, so both update kernels are timed, but for
+        // plans that are far off with the first)
         for (int supd = 0; supd <= 1; ++supd) {
           if (c->supd_mode != 0 && c->supd_mode != 1 + supd) continue;
           s.supd = supd;
-          consider(s, time_shape(c, s));
+          if (!(consider(s) < hopeless(true))) break;
         }
       }
     }
@@ -1367,7 +1415,7 @@ kmc_status autotune(kmc_ctx *c) {
       for (auto &t : near) {
         Shape s = t.second;
         s.supd = 1;
-        consider(s, time_shape(c, s));
+        consider(s);
       }
     }
   }
@@ -1384,7 +1432,7 @@ kmc_status autotune(kmc_ctx *c) {
     s.warps = 4;
     s.tile = 32;
     s.f64 = parts;
-    consider(s, time_shape(c, s));
+    consider(s);
   }
   // the whole period in clusters (tests: KMC_TUNE_CLUSTER, wherever it can run)
   bool clu_pin = false;
@@ -1394,7 +1442,7 @@ kmc_status autotune(kmc_ctx *c) {
     s.warps = 8;
     s.tile = 64;
     s.clu = 1;
-    consider(s, time_shape(c, s));
+    consider(s);
     clu_pin = std::getenv("KMC_TUNE_CLUSTER") != nullptr && !timed.empty() &&
               s == timed.back().second;
     if (clu_pin) {
@@ -1422,8 +1470,7 @@ kmc_status autotune(kmc_ctx *c) {
           s.chunk = ch;
           s.tpl = 1;
           s.rpl = rpl;
-          const float ms = time_shape(c, s);
-          consider(s, ms);
+          consider(s);
         }
       }
     }
@@ -1446,25 +1493,20 @@ kmc_status autotune(kmc_ctx *c) {
           s.tile = t;
           s.chunk = ch;
           s.tpl = tpl;
-          if (c->cl_mode != 2 && c->persist_mode != 2) {
-            const float ms = time_shape(c, s);
-            consider(s, ms);
-          }
+          if (c->cl_mode != 2 && c->persist_mode != 2) consider(s);
           // the same shape with each group's two parts as a two-CTA cluster
           // (time_shape fails unless every group has exactly two parts)
           if (c->fp32 && tpl == 1 && ch > 0 && c->cl_mode != 1 && c->persist_mode != 2) {
             Shape sc = s;
             sc.cl = 2;
-            const float mc = time_shape(c, sc);
-            consider(sc, mc);
+            consider(sc);
           }
           // the same shape as one persistent launch per period (time_shape
           // fails unless every item's block can be resident at once)
           if (c->fp32 && tpl == 1 && c->persist_mode != 1 && c->cl_mode != 2) {
             Shape sp = s;
             sp.persist = 1;
-            const float mp = time_shape(c, sp);
-            consider(sp, mp);
+            consider(sp);
           }
         }
       }
@@ -1486,7 +1528,7 @@ kmc_status autotune(kmc_ctx *c) {
     if (fin.size() > 1) {
       for (int r = 0; r < 2; ++r)
         for (auto &f : fin) {
-          const float ms = time_shape(c, f.second, 3);
+          const float ms = time_shape(c, f.second, std::numeric_limits<float>::infinity(), 3);
           show("finalist", f.second, ms);
           if (ms > 0.f && ms < f.first) f.first = ms;
         }
