@@ -92,3 +92,16 @@ def test_lysosomes_of_a_batch():
         np.testing.assert_allclose(kmc.kmc_local_concentration(ctx, q, 20), _oracle(lyss[q], 20),
                                    rtol=1e-13)
     kmc.kmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [2, 7, 8, 9, 33, 65])
+@pytest.mark.parametrize("prec", [kmc.KMC_FP64_PLAIN, kmc.KMC_FP32_MIXED])
+def test_small_samples(n, prec):
+    """About the size from which the grid serves (8 NPs): few cells, and ranks up to all
+    other NPs, which need the whole box."""
+    ly = _sample("random", n)
+    ctx = kmc.kmc_create([ly], prec, center=np.zeros(3))
+    for N in {1, max(1, n // 2), min(n - 1, 64)}:
+        np.testing.assert_allclose(kmc.kmc_local_concentration(ctx, 0, N), _oracle(ly, N),
+                                   rtol=1e-13)
+    kmc.kmc_destroy(ctx)
