@@ -112,16 +112,14 @@ def launch_info(kmc, ctx, lyss):
     ordered pair of its row group (whole cells, padding included), an
     off-diagonal item 28 packed operations per record and target, i.e. 14 lane
     operations per ordered pair, over its cells."""
-    warps, tile, chunk = kmc.kmc_tuning(ctx)
-    tpl = kmc.kmc_targets_per_lane(ctx)
-    rpl = kmc.kmc_replicas_per_lane(ctx)
-    form = kmc.kmc_pair_form(ctx)
+    shape = kmc.kmc_launch_shape(ctx)
+    warps, tile, chunk, tpl, rpl = (shape[k] for k in ("warps", "tile", "chunk", "tpl", "rpl"))
     n = [l.n for l in lyss]
     pairs = sum(v * (v - 1) for v in n)
     launch = {"warps": warps, "tile": tile, "chunk": chunk, "targets_per_lane": tpl,
               "replicas_per_lane": rpl}
-    if form == kmc.FORM_SYMMETRIC:
-        cells, cell = tpl // 2, kmc.KMC_CELL
+    if shape["sym_cells"]:
+        cells, cell = shape["sym_cells"], kmc.KMC_CELL
         gc = warps * cells
         items, upd, _, cut, _ = kmc.kmc_plan_sym(n, gc, chunk // cell)
         ops = 0
@@ -132,24 +130,25 @@ def launch_info(kmc, ctx, lyss):
             else:
                 ops += 14 * 2 * (gc * cell) * ((h1 - h0) * cell)
         chains = len(cut) - 1
-        block = kmc.kmc_sym_update(ctx) == 2
+        block = shape["sym_update"] == 1
         launch.update({"pair_form": "symmetric", "chains": chains, "update_items": len(upd),
                        "update": "block" if block else "warp"})
-        if chunk:  # 0: whole rows or balanced items
+        if shape["balanced"]:  # their number is the device's; the pairs are those of whole rows
+            launch["balanced"] = shape["balanced"]
+        else:
             launch["field_items"] = len(items)
         return {"launch": launch, "kernel": "kmc_field_sym<%d, %d> + kmc_update_sym%s<%d>" % (
                     warps, cells, "_block" if block else "", gc),
                 "lane_ops_per_pair": ops / pairs, "chains": chains,
                 "launches_per_period": lambda S: 2 * S * chains,
-                "key": (warps, tile, chunk, tpl, rpl, "sym") + (("block",) if block else ())}
-    if kmc.kmc_persistent(ctx) == 2:  # one cooperative launch per period, then the advance
+                "key": (warps, tile, chunk, tpl, rpl, "sym") + (("block",) if block else ()) +
+                (("balanced",) if shape["balanced"] else ())}
+    if shape["persistent"]:  # one cooperative launch per period, then the advance
         launch.update({"pair_form": "ordered", "chains": 1, "persistent": True})
         return {"launch": launch, "kernel": "kmc_persist_f32<%d>" % warps,
                 "lane_ops_per_pair": lane_ops_per_pair(rpl), "chains": 1,
                 "launches_per_period": lambda S: 1, "key": (warps, tile, chunk, tpl, rpl, "persist")}
-    if max(n) <= 512 and (warps, tile, chunk, tpl, rpl) == (8, 64, 0, 1, 1):
-        # the shape of a period in clusters (kmc_step_f32<8> can have it too: the count is
-        # the smaller of the two)
+    if shape["cluster_period"]:
         launch.update({"pair_form": "ordered", "chains": 1, "cluster_period": True})
         return {"launch": launch, "kernel": "kmc_cluster_f32<8>",
                 "lane_ops_per_pair": lane_ops_per_pair(rpl), "chains": 1,
@@ -821,13 +820,16 @@ def main():
         e1.record(stream)
         kmc.kmc_sync(c64)
         t64 = e0.elapsed_time(e1) / 1e3
-        w64, tl64, ch64 = kmc.kmc_tuning(c64)
-        form64 = "symmetric" if kmc.kmc_pair_form(c64) == kmc.FORM_SYMMETRIC else "ordered"
+        sh64 = kmc.kmc_launch_shape(c64)
+        launch64 = {k: sh64[k] for k in ("warps", "tile", "chunk")}
+        launch64["pair_form"] = "symmetric" if sh64["fp64_parts"] else "ordered"
+        if sh64["fp64_parts"]:
+            launch64["parts"] = sh64["fp64_parts"]
         units64 = n_np * S64 * per64
         fp64 = {"value": units64 / t64, "unit": UNIT,
                 "ms_per_step": 1e3 * t64 * units_per_step / units64,
                 "speedup_fp32_mixed": float(value / world / (units64 / t64)),
-                "launch": {"warps": w64, "tile": tl64, "chunk": ch64, "pair_form": form64}}
+                "launch": launch64}
         if not fp64_steps:
             sar64 = [kmc.kmc_read(c64, kmc.KMC_READ_SAR, l)[0] for l in range(len(lyss))]
             rel = abs(np.mean(sar32) - np.mean(sar64)) / abs(np.mean(sar64))
