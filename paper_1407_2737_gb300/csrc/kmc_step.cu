@@ -492,24 +492,34 @@ struct Decision {
   int nmin, flipped, near, bad, polished;
 };
 
-// e^x for an exponent x held in FP64: x log2(e) = n + f exactly split into an
-// integer n and a fraction f in [0, 1); 2^f in FP32, then scaled by 2^n. The
-// split adds 1.5 2^52 rounding down, which leaves floor in the low word, where
-// floor(), its conversions and ldexpf made a longer chain (0.4 to 1 % of a step).
-__device__ __forceinline__ float exp_fp64_arg(double x) {
+// 2^(y - shift) for an exponent y held in FP64 (yf: in FP32): y = n + f exactly split
+// into an integer n and a fraction f in [0, 1); 2^f in FP32, then scaled by
+// 2^(n - shift). The split adds 1.5 2^52 rounding down, which leaves floor in the low
+// word, where floor(), its conversions and ldexpf made a longer chain (0.4 to 1 % of
+// a step). y - shift is 121 at most.
+__device__ __forceinline__ float exp2_fp64_arg(double y, float yf, int shift) {
   constexpr double kShift = 6755399441055744.0;  // 1.5 2^52
-  const double y = x * 1.4426950408889634073599;  // log2(e)
-  const float yf = static_cast<float>(y);
-  if (yf < -160.0f) return 0.0f;
-  if (yf > 200.0f) return INFINITY;  // beyond FP32 (2^128 and more)
+  if (yf < static_cast<float>(shift - 160)) return 0.0f;
   const double t = __dadd_rd(y, kShift);
-  const int n = __double2loint(t);
+  const int n = __double2loint(t) - shift;
   const float r = exp2f(static_cast<float>(y - (t - kShift)));
   // r 2^n, r in [1, 2]: two exact scalings and one that rounds, as ldexpf's
   const int m = max(n, -126);
   const float lo = __int_as_float((max(n - m, -126) + 127) << 23);  // 2^(n - m) <= 1
-  if (m > 127) return INFINITY;
   return r * __int_as_float((m + 127) << 23) * lo;
+}
+
+// ea = e^xa and eb = e^xb in FP32, or both scaled down by one power of two where
+// FP32 does not hold them: their sum is then above 2^119, and (ea / sum) (1 - e^-sum)
+// is what it is for the unscaled ones. Beyond 2^(2^20) both are infinite.
+__device__ __forceinline__ void fp32_rates(double xa, double xb, float &ea, float &eb) {
+  constexpr double kLog2e = 1.4426950408889634073599;
+  const double ya = xa * kLog2e, yb = xb * kLog2e;
+  const float fa = static_cast<float>(ya), fb = static_cast<float>(yb), top = fmaxf(fa, fb);
+  const int shift = max(__float2int_rd(top) - 120, 0);
+  ea = exp2_fp64_arg(ya, fa, shift);
+  eb = exp2_fp64_arg(yb, fb, shift);
+  if (top > 1048576.0f) ea = eb = INFINITY;
 }
 
 // Steps v-vii for target t: basins, barrier (FP64 polish near the switching
@@ -611,8 +621,8 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
     if constexpr (MIXED) {
       // the exponent x in FP64; e^x = 2^n 2^f with n integral and the
       // fraction f in [0, 1) evaluated in FP32
-      const float ea = exp_fp64_arg(lognu0t - beta * dEa);
-      const float eb = exp_fp64_arg(lognu0t - beta * dEb);
+      float ea, eb;
+      fp32_rates(lognu0t - beta * dEa, lognu0t - beta * dEb, ea, eb);
       const float sum = ea + eb;
       P = (sum > 0.f) ? static_cast<double>((ea / sum) * (-expm1f(-sum))) : 0.0;
     } else {
@@ -621,9 +631,10 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
       P = 0.0;
       if (!exact_p) {
         // relative error of Pf below 1.2e-6: 2 ulp in each exponential, then
-        // the sum, the quotient, expm1 and the product. Where a rate or their sum
-        // exceeds FP32 the quotient is 0 or a NaN: not settled
-        const float ea = exp_fp64_arg(xa), eb = exp_fp64_arg(xb), sum = ea + eb;
+        // the sum, the quotient, expm1 and the product
+        float ea, eb;
+        fp32_rates(xa, xb, ea, eb);
+        const float sum = ea + eb;
         const float Pf = (sum > 0.f) ? (ea / sum) * (-expm1f(-sum)) : 0.f;
         const float uf = static_cast<float>(u);
         settled = isfinite(sum) && fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
