@@ -631,13 +631,14 @@ __device__ __forceinline__ Decision decide(const EpiShared<R> &sm, int t,
       P = 0.0;
       if (!exact_p) {
         // relative error of Pf below 1.2e-6: 2 ulp in each exponential, then
-        // the sum, the quotient, expm1 and the product
+        // the sum, the quotient, expm1 and the product; not a number where fp32_rates
+        // gives up, which is not settled
         float ea, eb;
         fp32_rates(xa, xb, ea, eb);
         const float sum = ea + eb;
         const float Pf = (sum > 0.f) ? (ea / sum) * (-expm1f(-sum)) : 0.f;
         const float uf = static_cast<float>(u);
-        settled = isfinite(sum) && fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
+        settled = fabsf(uf - Pf) > 4e-6f * Pf + 2e-7f * uf + 1.1e-9f;
         P = Pf;
       }
       if (!settled) {
