@@ -1169,9 +1169,9 @@ kmc_status capture_steps(kmc_ctx *c, const StepArgs &a, const Shape &sh, int ste
 // or a negative value on error. A candidate whose second launch alone took
 // longer than `hopeless` a step is given up with that time: most candidates are
 // 1.3 to 3 times slower than the best. First run of a size with all of them timed
-// in full and with this: 50 000 NPs 3.24 and 1.76 s, 96 lysosomes of about 1400
-// NPs 3.4 and 2.2 s, 8 x 2000 0.91 and 0.63 s, 8000 0.23 and 0.09 s, 1000 47 and
-// 45 ms, 100 7 and 4 ms.
+// in full and with this: 50 000 NPs 3.24 and 1.83 s, 96 lysosomes of about 1400
+// NPs 3.4 and 2.3 s, 8 x 2000 0.91 and 0.64 s, 8000 0.23 and 0.10 s, 1000 47 and
+// 49 ms, 100 7 and 4 ms.
 float time_shape(kmc_ctx *c, const Shape &s, float hopeless, int scale = 1) {
   const KeepError keep;
   if (set_items(c, s) != KMC_OK) return -1.f;
@@ -1251,11 +1251,11 @@ float time_shape(kmc_ctx *c, const Shape &s, float hopeless, int scale = 1) {
     ms /= reps * (gx ? graph_steps : 1);
     return ok;
   };
-  // (the wait leaves the GPU idle: a single launch is led by an untimed one again)
+  // (the wait leaves the GPU idle: single launches are led by two untimed ones again)
   const bool look = std::isfinite(hopeless);
   bool ok = !look || timed(1, 1);
   if (ok && (!look || ms < hopeless))
-    ok = timed(look ? (gx ? 0 : 1) : 2, (gx ? 2 : 5) * scale);
+    ok = timed(look && gx ? 0 : 2, (gx ? 2 : 5) * scale);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (gx) cudaGraphExecDestroy(gx);
@@ -1393,8 +1393,9 @@ kmc_status autotune(kmc_ctx *c) {
         s.sym = v[1];
         s.bal = bal;
         // (their targets gather more slots, so both update kernels are timed, but for
-        // plans that are far off with the first)
-        for (int supd = 0; supd <= 1; ++supd) {
+        // plans that are far off with a block per item: a warp takes 0.86 to 1.7 times
+        // its step)
+        for (int supd = 1; supd >= 0; --supd) {
           if (c->supd_mode != 0 && c->supd_mode != 1 + supd) continue;
           s.supd = supd;
           if (!(consider(s) < hopeless(true))) break;
