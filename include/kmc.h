@@ -441,7 +441,10 @@ kmc_status kmc_shell_profile(kmc_ctx *ctx, int32_t lys, double radius, int32_t n
  * volume-weighted mean m_z after each recorded step of every lysosome,
  * loop_M [n_lys][S * (periods - discard)] (host buffer of capacity cap;
  * KMC_ECAPACITY and *written = the size needed if too small). Starts from
- * m = +-easy axis with m_z >= 0, like kmc_create. Synchronous. */
+ * m = +-easy axis with m_z >= 0, like kmc_create. Synchronous. It allocates
+ * device memory for the call: what the NPs take and the wells of some steps,
+ * up to 64 MB, or of a whole period, up to 1 GB, if there are several; where
+ * that is refused, of fewer steps, with the same results. */
 kmc_status kmc_mean_run(const kmc_lysosome *lys, int32_t n_lys, const double *mu0Hmax,
                         int32_t n_amp, double f, int32_t steps_per_period, int32_t periods,
                         int32_t discard_periods, double *loop_M, int64_t cap,

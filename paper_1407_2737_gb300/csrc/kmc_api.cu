@@ -156,17 +156,17 @@ struct Shape {
   int cl = 0;
   // symmetric form's update kernel: 0 = one warp per update item, 1 = one block
   int supd = 0;
-  // symmetric form, the autotuner's alone: items of about equal work, bal waves of
+  // symmetric form (the autotuner or kmc_launch_shape): items of about equal work, bal waves of
   // the blocks that the SMs hold (chunk = 0); 0 = items of `chunk` source NPs
   int bal = 0;
   // 1: the whole field period as one persistent cooperative launch (FP32, one
   // target per lane) with a grid barrier after each step
   int persist = 0;
   // 1: the whole field period of lysosomes of up to 512 NPs as one launch, a
-  // thread-block cluster per lysosome (the autotuner's alone; FP32, warps = 8,
-  // chunk = 0)
+  // thread-block cluster per lysosome (the autotuner or kmc_launch_shape; FP32,
+  // warps = 8, tile = 64, chunk = 0)
   int clu = 0;
-  // symmetric form of FP64 contexts, the autotuner's alone: parts per cell pair
+  // symmetric form of FP64 contexts (the autotuner or kmc_launch_shape): parts per cell pair
   // (1, 2, 4, 8 or 16; warps = 4, tile = 32, chunk = 0); 0 = the ordered kernel
   int f64 = 0;
   bool operator==(const Shape &o) const {

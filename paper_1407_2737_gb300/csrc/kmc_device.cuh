@@ -204,8 +204,10 @@ __device__ __forceinline__ double rsqrt_seed(double x) {
 
 // 1/sqrt(r2), and 0 for r2 = 0 (a self pair, or two NPs at one point) or an
 // overflowed r2. The seed y has a short mantissa, so y y is exact and e = 1 -
-// r2 y^2 is rounded once; y (1 + e/2 + 3/8 e^2) leaves 5/16 e^3, far below the
-// rounding for a seed good to 2^-20.
+// r2 y^2 is rounded once; the binomial series (1 - e)^(-1/2) = 1 + e/2 + 3/8 e^2
+// + ..., cut there (Chebyshev's iteration for y^-2 = r2), leaves 5/16 e^3, far below the
+// rounding for a seed good to 2^-20. Fields of single pairs come out as the
+// oracle's do, 1e-15 off (sqrt and a division).
 __device__ __forceinline__ double rsqrt_pair(double r2) {
   const int hi = __double2hiint(r2);
   const bool none = (hi | __double2loint(r2)) == 0 || hi >= 0x7ff00000;

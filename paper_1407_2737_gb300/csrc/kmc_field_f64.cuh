@@ -16,8 +16,8 @@
 // shuffles with the reverse sums it has gathered. A warp shares nothing with
 // another, so a plan places an item on any SM: that is what small lysosomes
 // need, whose few target groups would otherwise keep a few SMs' FP64 pipes
-// busy while the others idle (100 NPs: 10 cell pairs, cut in 8 parts, run on
-// 80 SMs). A diagonal pair (g = h) runs its rotations 1 .. 31 forward only: 23
+// busy while the others idle (100 NPs: 10 cell pairs, cut in 16 parts, run on
+// every SM). A diagonal pair (g = h) runs its rotations 1 .. 31 forward only: 23
 // instructions per ordered pair. Every item writes its sums to its own slot, and
 // the update adds a target's slots in a fixed order: results are deterministic
 // and do not depend on the batch. Per step against the ordered
